@@ -28,30 +28,48 @@ bool factor_length(int L, LenPlan& pl)
     return rest == 1;
 }
 
-TileShape choose_tile(int L, size_t elem_bytes, int min_w, int max_w)
+static TileShape tile_of(int L, size_t elem_bytes, int LW, bool along_lines)
 {
     TileShape t;
-    // odd line stride (in elements) keeps the W-strided tile loads free of
-    // shared-memory bank conflicts for 8- and 16-byte elements
-    t.ld = (L % 2 == 0) ? L + 1 : L;
-    const size_t budget = 112 * 1024;  // two CTAs per SM
-    int W = max_w;
-    while (W > min_w && (2 * (size_t)W * t.ld + L) * elem_bytes > budget) W /= 2;
-    t.W = W;
-    t.smem = (2 * (size_t)W * t.ld + L) * elem_bytes;
+    t.LW = LW;
+    t.W = 1 << LW;
+    t.S = along_lines && t.W > 1 ? t.W + 1 : t.W;
+    t.smem = (2 * (size_t)t.S * L + L) * elem_bytes;
     return t;
 }
 
-TileShape plan_tile(const LenPlan& pl, size_t elem_bytes, int min_w, int max_w)
+static int floor_log2(int v)
+{
+    int l = 0;
+    while ((2 << l) <= v) l++;
+    return l;
+}
+
+TileShape choose_tile(int L, size_t elem_bytes, int min_w, int max_w, bool along_lines)
+{
+    const size_t budget = 112 * 1024;  // two CTAs per SM
+    int lw = floor_log2(max_w);
+    while ((1 << lw) > min_w && tile_of(L, elem_bytes, lw, along_lines).smem > budget) lw--;
+    return tile_of(L, elem_bytes, lw, along_lines);
+}
+
+TileShape plan_tile(const LenPlan& pl, size_t elem_bytes, int min_w, int max_w, bool along_lines)
 {
     if (pl.tile_w >= min_w && pl.tile_w <= max_w) {
-        TileShape t;
-        t.ld = (pl.L % 2 == 0) ? pl.L + 1 : pl.L;
-        t.W = pl.tile_w;
-        t.smem = (2 * (size_t)t.W * t.ld + pl.L) * elem_bytes;
+        const TileShape t = tile_of(pl.L, elem_bytes, floor_log2(pl.tile_w), along_lines);
         if (t.smem <= 200 * 1024) return t;
     }
-    return choose_tile(pl.L, elem_bytes, min_w, max_w);
+    return choose_tile(pl.L, elem_bytes, min_w, max_w, along_lines);
+}
+
+LenPlan with_magic(LenPlan pl)
+{
+    uint64_t Ns = 1;
+    for (int s = 0; s < pl.nst; s++) {
+        pl.mag[s] = Ns > 1 ? (uint32_t)(((1ull << 32) + Ns - 1) / Ns) : 0u;
+        Ns *= (uint64_t)pl.rad[s];
+    }
+    return pl;
 }
 
 TwiddleCache::~TwiddleCache()

@@ -1,14 +1,30 @@
 // fft.cuh -- batched 1-D FFT passes over one axis of a 3-D array.
 //
-// Each CTA stages a tile of W lines of length L in shared memory, runs a
-// mixed-radix Stockham FFT (radices 2, 3, 4, 5, 7, 8; the autosort variant
-// so no bit reversal is needed) through two ping-pong buffers, and writes
-// the tile back. Tiles of a strided axis are W lines that are adjacent in
-// memory, so every one of the L rows of the tile is a contiguous run of W
-// complex elements (coalesced); tiles of the contiguous axis are W whole
-// lines. Loads go through a "prologue" functor and stores through a "store"
-// functor, which is how the pointwise spectrum products, the real<->complex
-// packing and the normalisation epilogues are fused into the passes.
+// Each CTA stages a tile of W lines of length L in shared memory (W a power
+// of two), runs a mixed-radix Stockham FFT (radices 2, 3, 4, 5, 7, 8; the
+// autosort variant so no bit reversal is needed) through two ping-pong
+// buffers, and writes the tile back. Tiles of a strided axis are W lines
+// that are adjacent in memory, so every one of the L rows of the tile is a
+// contiguous run of W complex elements (coalesced); tiles of the contiguous
+// axis are W whole lines. Loads go through a "prologue" functor and stores
+// through a "store" functor, which is how the pointwise spectrum products,
+// the real<->complex packing and the normalisation epilogues are fused into
+// the passes.
+//
+// Index arithmetic is what bounds these kernels: the length is a run-time
+// value, and with lines stored one after another (element j of line w at
+// w ld + j) every load, butterfly and store divided by L, L / radix or W at
+// run time, 320 issued instructions per complex element and pass at 270 and
+// 315 against 56 in the register kernels. So the tile is kept transposed,
+// element j of line w at j S + w: the lanes of a warp take the W lines of a
+// butterfly first (shifts and masks; their twiddles are one broadcast read),
+// a strided tile is copied without any index change (S = W), and the one
+// quotient left per butterfly is a multiplication by a reciprocal from the
+// plan. Contiguous tiles use S = W + 1 (odd), which keeps their copies
+// along a line free of bank conflicts. Same schedules and arithmetic, the
+// same results; ttm_correlate of 126 x 270 x 315 (n = 4, FP64 local sums)
+// went from 8.24 to 6.64 ms, a batch of six sub-tomograms of 96 .. 176 per
+// axis x two templates from 12.90 to 8.65 ms.
 //
 // Direction DIR = -1 computes sum_j x_j exp(-2 pi i jk/L) (forward),
 // DIR = +1 the unnormalised inverse.
@@ -44,6 +60,7 @@ struct LenPlan {
     int nst;
     int rad[kMaxStages];
     const void* tw;
+    uint32_t mag[kMaxStages];  // ceil(2^32 / product of the radices before a stage), set by with_magic
     int tile_w = 0;   // lines per CTA of the shared-memory passes (0: default)
     int no_reg = 0;   // 1: use the shared-memory passes even where register kernels exist
 };
@@ -199,55 +216,56 @@ template <int RAD, int DIR, typename R> __device__ __forceinline__ void dft(cx<R
 
 // ----------------------------------------------------------- stages --
 
-// One Stockham stage of radix RAD on W lines (line stride ld) from `in` to
-// `out`. Ns = product of the radices of the earlier stages.
+// One Stockham stage of radix RAD on the W = 2^LW lines of a tile (element j
+// of line w at j S + w) from `in` to `out`. Ns = product of the radices of
+// the earlier stages, mag = ceil(2^32 / Ns) (j < 2^16, so the high word of
+// j mag is j / Ns exactly), step = L / (Ns RAD).
 template <int RAD, int DIR, typename R>
 __device__ __forceinline__ void stockham_stage(const cx<R>* __restrict__ in, cx<R>* __restrict__ out,
-                                               int L, int ld, int W, int Ns,
+                                               int L, int S, int LW, int Ns, uint32_t mag, int step,
                                                const cx<R>* __restrict__ tw)
 {
     const int nb = L / RAD;
-    const int total = nb * W;
-    const int step = L / (Ns * RAD);
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        int w = t / nb;
-        int j = t - w * nb;
-        int k = j % Ns;
-        const cx<R>* src = in + w * ld;
+    const int w = threadIdx.x & ((1 << LW) - 1);
+    for (int j = threadIdx.x >> LW; j < nb; j += blockDim.x >> LW) {
+        const int k = Ns > 1 ? j - (int)__umulhi((uint32_t)j, mag) * Ns : 0;
+        const cx<R>* src = in + j * S + w;
         cx<R> v[RAD];
 #pragma unroll
-        for (int r = 0; r < RAD; r++) v[r] = src[j + r * nb];
+        for (int r = 0; r < RAD; r++) v[r] = src[r * nb * S];
         if (Ns > 1) {
+            const cx<R>* tk = tw;
 #pragma unroll
             for (int r = 1; r < RAD; r++) {
-                cx<R> t_ = tw[r * k * step];
+                tk += k * step;
+                cx<R> t_ = *tk;
                 if (DIR > 0) t_.y = -t_.y;
                 v[r] = cmul(v[r], t_);
             }
         }
         dft<RAD, DIR, R>(v);
-        cx<R>* dst = out + w * ld;
-        int base = (j / Ns) * Ns * RAD + k;
+        cx<R>* dst = out + ((j - k) * RAD + k) * S + w;
 #pragma unroll
-        for (int r = 0; r < RAD; r++) dst[base + r * Ns] = v[r];
+        for (int r = 0; r < RAD; r++) dst[r * Ns * S] = v[r];
     }
 }
 
-// Full transform of the W lines in a (scratch b); returns the buffer that
+// Full transform of the 2^LW lines in a (scratch b); returns the buffer that
 // holds the result. Ends with __syncthreads().
 template <int DIR, typename R>
-__device__ cx<R>* smem_fft(cx<R>* a, cx<R>* b, int ld, int W, const LenPlan& pl, const cx<R>* tw)
+__device__ cx<R>* smem_fft(cx<R>* a, cx<R>* b, int S, int LW, const LenPlan& pl, const cx<R>* tw)
 {
-    int Ns = 1;
+    int Ns = 1, step = pl.L;
     const int L = pl.L;
     for (int s = 0; s < pl.nst; s++) {
+        const uint32_t mag = pl.mag[s];
         switch (pl.rad[s]) {
-            case 2: stockham_stage<2, DIR, R>(a, b, L, ld, W, Ns, tw); break;
-            case 3: stockham_stage<3, DIR, R>(a, b, L, ld, W, Ns, tw); break;
-            case 4: stockham_stage<4, DIR, R>(a, b, L, ld, W, Ns, tw); break;
-            case 5: stockham_stage<5, DIR, R>(a, b, L, ld, W, Ns, tw); break;
-            case 7: stockham_stage<7, DIR, R>(a, b, L, ld, W, Ns, tw); break;
-            default: stockham_stage<8, DIR, R>(a, b, L, ld, W, Ns, tw); break;
+            case 2: step /= 2; stockham_stage<2, DIR, R>(a, b, L, S, LW, Ns, mag, step, tw); break;
+            case 3: step /= 3; stockham_stage<3, DIR, R>(a, b, L, S, LW, Ns, mag, step, tw); break;
+            case 4: step /= 4; stockham_stage<4, DIR, R>(a, b, L, S, LW, Ns, mag, step, tw); break;
+            case 5: step /= 5; stockham_stage<5, DIR, R>(a, b, L, S, LW, Ns, mag, step, tw); break;
+            case 7: step /= 7; stockham_stage<7, DIR, R>(a, b, L, S, LW, Ns, mag, step, tw); break;
+            default: step /= 8; stockham_stage<8, DIR, R>(a, b, L, S, LW, Ns, mag, step, tw); break;
         }
         Ns *= pl.rad[s];
         __syncthreads();
@@ -309,71 +327,75 @@ struct StridedAxis {
 
 // ------------------------------------------------------------ kernels --
 
-// Shared memory: 2 * W * ld + L complex elements.
-template <typename R, int DIR, class Pro, class Store, typename In = cx<R>>
-__global__ void __launch_bounds__(256) k_fft_strided(const In* __restrict__ in, StridedAxis ax, LenPlan pl,
-                                                     int W, int ld, Pro pro, Store store)
+constexpr int kSmemFftThreads = 256;
+
+// Stages elements x0, x0 + G, ... < n of one line with kLoadBatch global
+// loads issued before any of their shared-memory stores (see stage_tile)
+template <typename T, class Get, class Put>
+__device__ __forceinline__ void stage_line(int x0, int G, int n, Get get, Put put)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx<R>* bufa = reinterpret_cast<cx<R>*>(smem_raw);
-    cx<R>* bufb = bufa + W * ld;
-    cx<R>* tws = bufb + W * ld;
-    const int64_t tiles_per_outer = (ax.inner + W - 1) / W;
-    const int64_t o = blockIdx.x / tiles_per_outer;
-    const int64_t i0 = (blockIdx.x - o * tiles_per_outer) * W;
-    const int L = pl.L;
-    load_twiddles<R>(tws, pl);
-    stage_tile<cx<R>>(
-        W * L,
-        [&](int idx) {
-            const int j = idx / W, w = idx - j * W;
-            const int64_t i = i0 + w;
-            return i < ax.inner ? pro(load_cx(in[o * ax.os + i + (int64_t)j * ax.s]), o, i, j) : mk<R>(0, 0);
-        },
-        [&](int idx, cx<R> v) {
-            const int j = idx / W, w = idx - j * W;
-            bufa[w * ld + j] = v;
-        });
-    __syncthreads();
-    cx<R>* res = smem_fft<DIR, R>(bufa, bufb, ld, W, pl, tws);
-    for (int idx = threadIdx.x; idx < W * L; idx += blockDim.x) {
-        int j = idx / W, w = idx - j * W;
-        int64_t i = i0 + w;
-        if (i < ax.inner) store(res[w * ld + j], o, i, j);
+    for (int base = x0; base < n; base += kLoadBatch * G) {
+        T v[kLoadBatch];
+#pragma unroll
+        for (int u = 0; u < kLoadBatch; u++)
+            if (base + u * G < n) v[u] = get(base + u * G);
+#pragma unroll
+        for (int u = 0; u < kLoadBatch; u++)
+            if (base + u * G < n) put(base + u * G, v[u]);
     }
 }
 
-// Contiguous lines: line l has elements l*L + j (l < nlines). The functors
-// get (o = l, i = 0, j).
-template <typename R, int DIR, class Pro, class Store>
-__global__ void __launch_bounds__(256) k_fft_contig(const cx<R>* __restrict__ in, int64_t nlines, LenPlan pl,
-                                                    int W, int ld, Pro pro, Store store)
+// Shared memory: 2 * L * W + L complex elements (W = 2^LW lines, S = W).
+template <typename R, int DIR, class Pro, class Store, typename In = cx<R>>
+__global__ void __launch_bounds__(kSmemFftThreads) k_fft_strided(const In* __restrict__ in, StridedAxis ax, LenPlan pl,
+                                                     int LW, Pro pro, Store store)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int L = pl.L, W = 1 << LW;
     cx<R>* bufa = reinterpret_cast<cx<R>*>(smem_raw);
-    cx<R>* bufb = bufa + W * ld;
-    cx<R>* tws = bufb + W * ld;
-    const int64_t l0 = (int64_t)blockIdx.x * W;
-    const int L = pl.L;
+    cx<R>* bufb = bufa + L * W;
+    cx<R>* tws = bufb + L * W;
+    const int64_t tiles_per_outer = (ax.inner + W - 1) >> LW;
+    const int64_t o = blockIdx.x / tiles_per_outer;
+    const int64_t i = ((blockIdx.x - o * tiles_per_outer) << LW) + (threadIdx.x & (W - 1));
+    const bool act = i < ax.inner;
     load_twiddles<R>(tws, pl);
+    const In* src = in + o * ax.os + i;
     stage_tile<cx<R>>(
         W * L,
         [&](int idx) {
-            const int w = idx / L, j = idx - w * L;
-            const int64_t l = l0 + w;
-            return l < nlines ? pro(in[l * L + j], l, 0, j) : mk<R>(0, 0);
+            const int j = idx >> LW;
+            return act ? pro(load_cx(src[(int64_t)j * ax.s]), o, i, j) : mk<R>(0, 0);
         },
-        [&](int idx, cx<R> v) {
-            const int w = idx / L, j = idx - w * L;
-            bufa[w * ld + j] = v;
-        });
+        [&](int idx, cx<R> v) { bufa[idx] = v; });
     __syncthreads();
-    cx<R>* res = smem_fft<DIR, R>(bufa, bufb, ld, W, pl, tws);
-    for (int idx = threadIdx.x; idx < W * L; idx += blockDim.x) {
-        int w = idx / L, j = idx - w * L;
-        int64_t l = l0 + w;
-        if (l < nlines) store(res[w * ld + j], l, 0, j);
-    }
+    cx<R>* res = smem_fft<DIR, R>(bufa, bufb, W, LW, pl, tws);
+    if (act)
+        for (int idx = threadIdx.x; idx < W * L; idx += kSmemFftThreads) store(res[idx], o, i, idx >> LW);
+}
+
+// Contiguous lines: line l has elements l*L + j (l < nlines). The functors
+// get (o = l, i = 0, j). 256 / W consecutive threads work on one line.
+template <typename R, int DIR, class Pro, class Store>
+__global__ void __launch_bounds__(kSmemFftThreads) k_fft_contig(const cx<R>* __restrict__ in, int64_t nlines, LenPlan pl,
+                                                    int LW, int S, Pro pro, Store store)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int L = pl.L, G = kSmemFftThreads >> LW;
+    cx<R>* bufa = reinterpret_cast<cx<R>*>(smem_raw);
+    cx<R>* bufb = bufa + L * S;
+    cx<R>* tws = bufb + L * S;
+    const int w = threadIdx.x / G, x0 = threadIdx.x & (G - 1);
+    const int64_t l = ((int64_t)blockIdx.x << LW) + w;
+    const bool act = l < nlines;
+    load_twiddles<R>(tws, pl);
+    stage_line<cx<R>>(
+        x0, G, L, [&](int j) { return act ? pro(in[l * L + j], l, 0, j) : mk<R>(0, 0); },
+        [&](int j, cx<R> v) { bufa[j * S + w] = v; });
+    __syncthreads();
+    cx<R>* res = smem_fft<DIR, R>(bufa, bufb, S, LW, pl, tws);
+    if (act)
+        for (int j = x0; j < L; j += G) store(res[j * S + w], l, 0, j);
 }
 
 // Forward real-to-complex along the contiguous axis, two real rows per
@@ -381,30 +403,26 @@ __global__ void __launch_bounds__(256) k_fft_contig(const cx<R>* __restrict__ in
 // B(k) = (Z(k) - conj Z(-k)) / (2i), k in [0, X/2]. `src(row, x)` yields the
 // real input (so padding / wrapping / type conversion fuse into the load).
 template <typename R, class Src>
-__global__ void __launch_bounds__(256) k_r2c_rows(Src src, int64_t nrows, cx<R>* __restrict__ out, LenPlan pl,
-                                                  int W, int ld)
+__global__ void __launch_bounds__(kSmemFftThreads) k_r2c_rows(Src src, int64_t nrows, cx<R>* __restrict__ out, LenPlan pl,
+                                                  int LW, int S)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int X = pl.L, Xh = X / 2 + 1, G = kSmemFftThreads >> LW;
     cx<R>* bufa = reinterpret_cast<cx<R>*>(smem_raw);
-    cx<R>* bufb = bufa + W * ld;
-    cx<R>* tws = bufb + W * ld;
-    const int X = pl.L, Xh = X / 2 + 1;
-    const int64_t r0 = (int64_t)blockIdx.x * 2 * W;
+    cx<R>* bufb = bufa + X * S;
+    cx<R>* tws = bufb + X * S;
+    const int w = threadIdx.x / G, x0 = threadIdx.x & (G - 1);
+    const int64_t ra = ((int64_t)blockIdx.x << (LW + 1)) + 2 * w, rb = ra + 1;
     load_twiddles<R>(tws, pl);
-    for (int idx = threadIdx.x; idx < W * X; idx += blockDim.x) {
-        int w = idx / X, x = idx - w * X;
-        int64_t ra = r0 + 2 * w, rb = ra + 1;
-        R a = ra < nrows ? src(ra, x) : (R)0;
-        R b = rb < nrows ? src(rb, x) : (R)0;
-        bufa[w * ld + x] = mk<R>(a, b);
-    }
+    stage_line<cx<R>>(
+        x0, G, X,
+        [&](int x) { return mk<R>(ra < nrows ? src(ra, x) : (R)0, rb < nrows ? src(rb, x) : (R)0); },
+        [&](int x, cx<R> v) { bufa[x * S + w] = v; });
     __syncthreads();
-    cx<R>* res = smem_fft<-1, R>(bufa, bufb, ld, W, pl, tws);
-    for (int idx = threadIdx.x; idx < W * Xh; idx += blockDim.x) {
-        int w = idx / Xh, k = idx - w * Xh;
-        int64_t ra = r0 + 2 * w, rb = ra + 1;
-        cx<R> zk = res[w * ld + k];
-        cx<R> zn = res[w * ld + (k == 0 ? 0 : X - k)];
+    cx<R>* res = smem_fft<-1, R>(bufa, bufb, S, LW, pl, tws);
+    for (int k = x0; k < Xh; k += G) {
+        cx<R> zk = res[k * S + w];
+        cx<R> zn = res[(k == 0 ? 0 : X - k) * S + w];
         // A = (zk + conj zn)/2 ; B = (zk - conj zn)/(2i)
         cx<R> A = mk<R>((zk.x + zn.x) * (R)0.5, (zk.y - zn.y) * (R)0.5);
         cx<R> d = mk<R>(zk.x - zn.x, zk.y + zn.y);
@@ -418,45 +436,51 @@ __global__ void __launch_bounds__(256) k_r2c_rows(Src src, int64_t nrows, cx<R>*
 // per complex line: Z(k) = A(k) + i B(k) for k <= X/2 and
 // Z(k) = conj A(X-k) + i conj B(X-k) above, with the imaginary parts of the
 // k = 0 (and k = X/2 for even X) bins dropped as a C2R transform does;
-// IFFT(Z) = a + i b. `sink(row, x, value)` consumes the real outputs
-// (normalisation / max epilogues). `in` may be offset per blockIdx.y by
-// in_batch_stride for batched use; the sink gets blockIdx.y via `batch`.
+// IFFT(Z) = a + i b. `sink(batch, row, x, value)` consumes the real outputs
+// (normalisation / max epilogues); nbatch arrays of nrows rows follow each
+// other in `in`.
 template <typename R, class Sink, typename In = cx<R>>
-__global__ void __launch_bounds__(256) k_c2r_rows(const In* __restrict__ in, int64_t nrows, Sink sink,
-                                                  LenPlan pl, int W, int ld, int nbatch)
+__global__ void __launch_bounds__(kSmemFftThreads) k_c2r_rows(const In* __restrict__ in, int64_t nrows, Sink sink,
+                                                  LenPlan pl, int LW, int S, int nbatch)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int X = pl.L, Xh = X / 2 + 1, G = kSmemFftThreads >> LW;
     cx<R>* bufa = reinterpret_cast<cx<R>*>(smem_raw);
-    cx<R>* bufb = bufa + W * ld;
-    cx<R>* tws = bufb + W * ld;
-    const int X = pl.L, Xh = X / 2 + 1;
+    cx<R>* bufb = bufa + X * S;
+    cx<R>* tws = bufb + X * S;
     // batch index fastest so that the CTAs sharing rows (and the rows of any
     // per-voxel factor the sink reads) run together
     const int batch = blockIdx.x % nbatch;
     const int64_t tile = blockIdx.x / nbatch;
-    const int64_t r0 = tile * 2 * W;
-    const In* src = in + (int64_t)batch * nrows * Xh;
+    const int w = threadIdx.x / G, x0 = threadIdx.x & (G - 1);
+    const int64_t ra = (tile << (LW + 1)) + 2 * w, rb = ra + 1;
+    const bool va = ra < nrows, vb = rb < nrows;
+    const In* ba = in + ((int64_t)batch * nrows + ra) * Xh;
+    const In* bb = ba + Xh;
     load_twiddles<R>(tws, pl);
-    for (int idx = threadIdx.x; idx < W * Xh; idx += blockDim.x) {
-        int w = idx / Xh, k = idx - w * Xh;
-        int64_t ra = r0 + 2 * w, rb = ra + 1;
-        cx<R> A = ra < nrows ? load_cx(src[ra * Xh + k]) : mk<R>(0, 0);
-        cx<R> B = rb < nrows ? load_cx(src[rb * Xh + k]) : mk<R>(0, 0);
-        if (k == 0 || (2 * k == X)) { A.y = 0; B.y = 0; }
-        // Z(k) = A + iB
-        bufa[w * ld + k] = mk<R>(A.x - B.y, A.y + B.x);
-        // Z(X-k) = conj A + i conj B, for the bins not covered above
-        int kk = X - k;
-        if (k >= 1 && kk >= Xh) bufa[w * ld + kk] = mk<R>(A.x + B.y, -A.y + B.x);
-    }
+    struct Pair { cx<R> A, B; };
+    stage_line<Pair>(
+        x0, G, Xh,
+        [&](int k) {
+            Pair p;
+            p.A = va ? load_cx(ba[k]) : mk<R>(0, 0);
+            p.B = vb ? load_cx(bb[k]) : mk<R>(0, 0);
+            return p;
+        },
+        [&](int k, Pair p) {
+            if (k == 0 || (2 * k == X)) { p.A.y = 0; p.B.y = 0; }
+            // Z(k) = A + iB
+            bufa[k * S + w] = mk<R>(p.A.x - p.B.y, p.A.y + p.B.x);
+            // Z(X-k) = conj A + i conj B, for the bins not covered above
+            const int kk = X - k;
+            if (k >= 1 && kk >= Xh) bufa[kk * S + w] = mk<R>(p.A.x + p.B.y, -p.A.y + p.B.x);
+        });
     __syncthreads();
-    cx<R>* res = smem_fft<+1, R>(bufa, bufb, ld, W, pl, tws);
-    for (int idx = threadIdx.x; idx < W * X; idx += blockDim.x) {
-        int w = idx / X, x = idx - w * X;
-        int64_t ra = r0 + 2 * w, rb = ra + 1;
-        cx<R> v = res[w * ld + x];
-        if (ra < nrows) sink(batch, ra, x, v.x);
-        if (rb < nrows) sink(batch, rb, x, v.y);
+    cx<R>* res = smem_fft<+1, R>(bufa, bufb, S, LW, pl, tws);
+    for (int x = x0; x < X; x += G) {
+        const cx<R> v = res[x * S + w];
+        if (va) sink(batch, ra, x, v.x);
+        if (vb) sink(batch, rb, x, v.y);
     }
 }
 
@@ -465,16 +489,19 @@ __global__ void __launch_bounds__(256) k_c2r_rows(const In* __restrict__ in, int
 // Radix schedule for L (7-smooth); returns false otherwise.
 bool factor_length(int L, LenPlan& pl);
 
-// Tile width (lines per CTA) and padded line stride for a pass of length L
-// in precision R, and its dynamic shared memory in bytes.
+// Tile of a shared-memory pass of length L: W = 2^LW lines per CTA, element
+// stride S (W, or W + 1 for tiles copied along their lines), and its
+// dynamic shared memory in bytes.
 struct TileShape {
-    int W, ld;
+    int W, LW, S;
     size_t smem;
 };
-TileShape choose_tile(int L, size_t elem_bytes, int min_w, int max_w);
-// the plan's tuned tile width if it has one (within the shared-memory
-// budget), else choose_tile
-TileShape plan_tile(const LenPlan& pl, size_t elem_bytes, int min_w, int max_w);
+TileShape choose_tile(int L, size_t elem_bytes, int min_w, int max_w, bool along_lines);
+// the plan's tuned tile width if it has one (rounded down to a power of two,
+// within the shared-memory budget), else choose_tile
+TileShape plan_tile(const LenPlan& pl, size_t elem_bytes, int min_w, int max_w, bool along_lines);
+// the plan with the reciprocals that its schedule needs
+LenPlan with_magic(LenPlan pl);
 
 }  // namespace ttm
 
@@ -510,12 +537,12 @@ template <typename R, int DIR, class Pro, class Store, typename In = cx<R>>
 inline void launch_strided(const In* in, StridedAxis ax, const LenPlan& pl, Pro pro, Store store,
                            cudaStream_t st)
 {
-    TileShape ts = plan_tile(pl, sizeof(cx<R>), 4, 16);
+    TileShape ts = plan_tile(pl, sizeof(cx<R>), 4, 16, false);
     auto k = k_fft_strided<R, DIR, Pro, Store, In>;
     set_smem(k, ts.smem);
     int64_t grid = ax.outer * ceil_div(ax.inner, ts.W);
     TTM_REQUIRE(grid < (1ll << 31), E_SHAPE, "strided pass grid too large");
-    k<<<(unsigned)grid, 256, ts.smem, st>>>(in, ax, pl, ts.W, ts.ld, pro, store);
+    k<<<(unsigned)grid, kSmemFftThreads, ts.smem, st>>>(in, ax, with_magic(pl), ts.LW, pro, store);
     TTM_LAUNCH_CHECK();
 }
 
@@ -523,22 +550,22 @@ template <typename R, int DIR, class Pro, class Store>
 inline void launch_contig(const cx<R>* in, int64_t nlines, const LenPlan& pl, Pro pro, Store store,
                           cudaStream_t st)
 {
-    TileShape ts = plan_tile(pl, sizeof(cx<R>), 1, 8);
+    TileShape ts = plan_tile(pl, sizeof(cx<R>), 1, 8, true);
     auto k = k_fft_contig<R, DIR, Pro, Store>;
     set_smem(k, ts.smem);
     int64_t grid = ceil_div(nlines, ts.W);
-    k<<<(unsigned)grid, 256, ts.smem, st>>>(in, nlines, pl, ts.W, ts.ld, pro, store);
+    k<<<(unsigned)grid, kSmemFftThreads, ts.smem, st>>>(in, nlines, with_magic(pl), ts.LW, ts.S, pro, store);
     TTM_LAUNCH_CHECK();
 }
 
 template <typename R, class Src>
 inline void launch_r2c_rows(Src src, int64_t nrows, cx<R>* out, const LenPlan& pl, cudaStream_t st)
 {
-    TileShape ts = choose_tile(pl.L, sizeof(cx<R>), 1, 8);
+    TileShape ts = choose_tile(pl.L, sizeof(cx<R>), 1, 8, true);
     auto k = k_r2c_rows<R, Src>;
     set_smem(k, ts.smem);
     int64_t grid = ceil_div(nrows, 2 * ts.W);
-    k<<<(unsigned)grid, 256, ts.smem, st>>>(src, nrows, out, pl, ts.W, ts.ld);
+    k<<<(unsigned)grid, kSmemFftThreads, ts.smem, st>>>(src, nrows, out, with_magic(pl), ts.LW, ts.S);
     TTM_LAUNCH_CHECK();
 }
 
@@ -546,12 +573,12 @@ template <typename R, class Sink, typename In = cx<R>>
 inline void launch_c2r_rows(const In* in, int64_t nrows, Sink sink, const LenPlan& pl, int nbatch,
                             cudaStream_t st)
 {
-    TileShape ts = plan_tile(pl, sizeof(cx<R>), 1, 8);
+    TileShape ts = plan_tile(pl, sizeof(cx<R>), 1, 8, true);
     auto k = k_c2r_rows<R, Sink, In>;
     set_smem(k, ts.smem);
     int64_t grid = ceil_div(nrows, 2 * ts.W) * nbatch;
     TTM_REQUIRE(grid < (1ll << 31), E_SHAPE, "c2r pass grid too large");
-    k<<<(unsigned)grid, 256, ts.smem, st>>>(in, nrows, sink, pl, ts.W, ts.ld, nbatch);
+    k<<<(unsigned)grid, kSmemFftThreads, ts.smem, st>>>(in, nrows, sink, with_magic(pl), ts.LW, ts.S, nbatch);
     TTM_LAUNCH_CHECK();
 }
 

@@ -212,7 +212,7 @@ const TuneRec& tune_length(ttm_ctx* ctx, int L)
             std::copy(sch.begin(), sch.end(), pl.rad);
             for (int W : {4, 8, 16}) {
                 pl.tile_w = W;
-                if (plan_tile(pl, sizeof(float2), 4, 16).W != W) continue;
+                if (plan_tile(pl, sizeof(float2), 4, 16, false).W != W) continue;
                 const double t = time_pass(buf.as<float2>(), pl, st, e0, e1);
                 if (t < best.us_line) {
                     best.us_line = t;

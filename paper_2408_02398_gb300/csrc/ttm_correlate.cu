@@ -42,56 +42,53 @@ __global__ void k_spec_store(const double2* __restrict__ src, int64_t n, double 
 }
 
 // Fused z pass. Columns c in [0, ncols) (ncols = Y * Xh) are the (ky, kx)
-// pairs; element z of column c is at z * ncols + c. One CTA owns W adjacent
-// columns. Shared memory: 3 * W * ld + Z complex.
+// pairs; element z of column c is at z * ncols + c. One CTA owns W = 2^LW
+// adjacent columns, kept as [z][w] (see fft.cuh). Shared memory:
+// 3 * W * Z + Z complex.
 template <typename TS, typename TW>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kSmemFftThreads)
 k_zcorr(const float2* __restrict__ G, const TS* __restrict__ spec, int K, int tzn, int cz, int64_t ncols,
-        TW* __restrict__ out, LenPlan pl, int W, int ld, const float* __restrict__ gmax, float oscale)
+        TW* __restrict__ out, LenPlan pl, int LW, const float* __restrict__ gmax, float oscale)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int Z = pl.L, W = 1 << LW;
     float2* gs = reinterpret_cast<float2*>(smem_raw);
-    float2* bufa = gs + W * ld;
-    float2* bufb = bufa + W * ld;
-    float2* tws = bufb + W * ld;
-    const int Z = pl.L;
-    const int64_t c0 = (int64_t)blockIdx.x * W;
+    float2* bufa = gs + W * Z;
+    float2* bufb = bufa + W * Z;
+    float2* tws = bufb + W * Z;
+    const int64_t c = ((int64_t)blockIdx.x << LW) + (threadIdx.x & (W - 1));
+    const bool act = c < ncols;
     load_twiddles<float>(tws, pl);
     const float gsc = (gmax && *gmax > 0.f) ? 1.f / *gmax : 1.f;
-    for (int idx = threadIdx.x; idx < W * Z; idx += blockDim.x) {
-        int z = idx / W, w = idx - z * W;
-        int64_t c = c0 + w;
-        gs[w * ld + z] = c < ncols ? cscale(G[(int64_t)z * ncols + c], gsc) : make_float2(0.f, 0.f);
-    }
+    stage_tile<float2>(
+        W * Z,
+        [&](int idx) {
+            return act ? cscale(G[(int64_t)(idx >> LW) * ncols + c], gsc) : make_float2(0.f, 0.f);
+        },
+        [&](int idx, float2 v) { gs[idx] = v; });
     const int64_t comp_stride = (int64_t)tzn * ncols;
     const int64_t out_stride = (int64_t)Z * ncols;
     for (int a = 0; a < K; a++) {
         // template rows j land on z = (j - cz) mod Z, i.e. j = (z + cz) mod Z
-        const TS* sp = spec + a * comp_stride;
-        for (int idx = threadIdx.x; idx < W * Z; idx += blockDim.x) {
-            int z = idx / W, w = idx - z * W;
-            int64_t c = c0 + w;
-            int j = z + cz;
-            if (j >= Z) j -= Z;
-            float2 v = make_float2(0.f, 0.f);
-            if (j < tzn && c < ncols) v = load_cx(sp[(int64_t)j * ncols + c]);
-            bufa[w * ld + z] = v;
-        }
+        const TS* sp = spec + a * comp_stride + c;
+        stage_tile<float2>(
+            W * Z,
+            [&](int idx) {
+                int j = (idx >> LW) + cz;
+                if (j >= Z) j -= Z;
+                return act && j < tzn ? load_cx(sp[(int64_t)j * ncols]) : make_float2(0.f, 0.f);
+            },
+            [&](int idx, float2 v) { bufa[idx] = v; });
         __syncthreads();
-        float2* p = smem_fft<-1, float>(bufa, bufb, ld, W, pl, tws);
+        float2* p = smem_fft<-1, float>(bufa, bufb, W, LW, pl, tws);
         float2* q = (p == bufa) ? bufb : bufa;
-        for (int idx = threadIdx.x; idx < W * Z; idx += blockDim.x) {
-            int w = idx / Z, z = idx - w * Z;
-            p[w * ld + z] = cmulconj(gs[w * ld + z], p[w * ld + z]);
-        }
+        for (int idx = threadIdx.x; idx < W * Z; idx += kSmemFftThreads) p[idx] = cmulconj(gs[idx], p[idx]);
         __syncthreads();
-        float2* r = smem_fft<+1, float>(p, q, ld, W, pl, tws);
-        TW* o = out + a * out_stride;
-        for (int idx = threadIdx.x; idx < W * Z; idx += blockDim.x) {
-            int z = idx / W, w = idx - z * W;
-            int64_t c = c0 + w;
-            if (c < ncols) store_cx(o + (int64_t)z * ncols + c, cscale(r[w * ld + z], oscale));
-        }
+        float2* r = smem_fft<+1, float>(p, q, W, LW, pl, tws);
+        TW* o = out + a * out_stride + c;
+        if (act)
+            for (int idx = threadIdx.x; idx < W * Z; idx += kSmemFftThreads)
+                store_cx(o + (int64_t)(idx >> LW) * ncols, cscale(r[idx], oscale));
         __syncthreads();
     }
 }
@@ -185,13 +182,16 @@ void launch_zcorr(const float2* G, const TS* spec, int K, int tzn, int cz, int64
     if (dw && launch_zcorr_tma(G, spec, K, tzn, cz, ncols, out, pz, gmax, oscale, *dw, st)) return;
     if (launch_zcorr_fs(G, spec, K, tzn, cz, ncols, out, pz, gmax, oscale, st)) return;
     const int Z = pz.L;
-    const int ld = (Z % 2 == 0) ? Z + 1 : Z;
-    int W = (pz.tile_w >= 2 && pz.tile_w <= 16) ? pz.tile_w : 16;
-    while (W > 2 && (3 * (size_t)W * ld + Z) * sizeof(float2) > 112 * 1024) W /= 2;
-    size_t smem = (3 * (size_t)W * ld + Z) * sizeof(float2);
+    int LW = 4;
+    if (pz.tile_w >= 2 && pz.tile_w <= 16)
+        while ((1 << LW) > pz.tile_w) LW--;
+    auto bytes = [&](int lw) { return ((3ull << lw) * Z + Z) * sizeof(float2); };
+    while (LW > 1 && bytes(LW) > 112 * 1024) LW--;
+    const size_t smem = bytes(LW);
     set_smem(k_zcorr<TS, TW>, smem);
-    int64_t grid = ceil_div(ncols, W);
-    k_zcorr<TS, TW><<<(unsigned)grid, 256, smem, st>>>(G, spec, K, tzn, cz, ncols, out, pz, W, ld, gmax, oscale);
+    const int64_t grid = ceil_div(ncols, 1 << LW);
+    k_zcorr<TS, TW><<<(unsigned)grid, kSmemFftThreads, smem, st>>>(G, spec, K, tzn, cz, ncols, out, with_magic(pz), LW,
+                                                                   gmax, oscale);
     TTM_LAUNCH_CHECK();
 }
 

@@ -301,42 +301,29 @@ struct StoreWDF {
 // double-float kernels inside the instruction cache). One read and one
 // write of the (g, g^2) spectrum instead of two each.
 template <typename R, class Mask>
-__global__ void __launch_bounds__(256)
-k_zmask(cx<R>* __restrict__ zd, int64_t ncols, LenPlan pl, int W, int ld, Mask mask)
+__global__ void __launch_bounds__(kSmemFftThreads)
+k_zmask(cx<R>* __restrict__ zd, int64_t ncols, LenPlan pl, int LW, Mask mask)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int Z = pl.L, W = 1 << LW;
     cx<R>* bufa = reinterpret_cast<cx<R>*>(smem_raw);
-    cx<R>* bufb = bufa + W * ld;
-    cx<R>* tws = bufb + W * ld;
-    const int Z = pl.L;
-    const int64_t c0 = (int64_t)blockIdx.x * W;
+    cx<R>* bufb = bufa + W * Z;
+    cx<R>* tws = bufb + W * Z;
+    const int64_t c = ((int64_t)blockIdx.x << LW) + (threadIdx.x & (W - 1));
+    const bool act = c < ncols;
     load_twiddles<R>(tws, pl);
     stage_tile<cx<R>>(
-        W * Z,
-        [&](int idx) {
-            const int z = idx / W, w = idx - z * W;
-            const int64_t c = c0 + w;
-            return c < ncols ? zd[(int64_t)z * ncols + c] : mk<R>(0, 0);
-        },
-        [&](int idx, cx<R> v) {
-            const int z = idx / W, w = idx - z * W;
-            bufa[w * ld + z] = v;
-        });
+        W * Z, [&](int idx) { return act ? zd[(int64_t)(idx >> LW) * ncols + c] : mk<R>(0, 0); },
+        [&](int idx, cx<R> v) { bufa[idx] = v; });
     __syncthreads();
-    cx<R>* p = smem_fft<-1, R>(bufa, bufb, ld, W, pl, tws);
+    cx<R>* p = smem_fft<-1, R>(bufa, bufb, W, LW, pl, tws);
     cx<R>* q = (p == bufa) ? bufb : bufa;
-    for (int idx = threadIdx.x; idx < W * Z; idx += blockDim.x) {
-        const int kz = idx / W, w = idx - kz * W;
-        const int64_t c = c0 + w;
-        if (c < ncols) p[w * ld + kz] = mask(p[w * ld + kz], 0, c, kz);
-    }
+    if (act)
+        for (int idx = threadIdx.x; idx < W * Z; idx += kSmemFftThreads) p[idx] = mask(p[idx], 0, c, idx >> LW);
     __syncthreads();
-    cx<R>* r = smem_fft<+1, R>(p, q, ld, W, pl, tws);
-    for (int idx = threadIdx.x; idx < W * Z; idx += blockDim.x) {
-        const int z = idx / W, w = idx - z * W;
-        const int64_t c = c0 + w;
-        if (c < ncols) zd[(int64_t)z * ncols + c] = r[w * ld + z];
-    }
+    cx<R>* r = smem_fft<+1, R>(p, q, W, LW, pl, tws);
+    if (act)
+        for (int idx = threadIdx.x; idx < W * Z; idx += kSmemFftThreads) zd[(int64_t)(idx >> LW) * ncols + c] = r[idx];
 }
 
 template <typename R, class Mask>
@@ -350,13 +337,13 @@ static void launch_zmask(cx<R>* zd, int64_t ncols, const LenPlan& pz, Mask mask,
         }
     }
     const int Z = pz.L;
-    const int ld = Z | 1;
-    int W = 16;
-    while (W > 2 && (2 * (size_t)W * ld + Z) * sizeof(cx<R>) > 110 * 1024) W /= 2;
-    const size_t smem = (2 * (size_t)W * ld + Z) * sizeof(cx<R>);
+    auto bytes = [&](int lw) { return ((2ull << lw) * Z + Z) * sizeof(cx<R>); };
+    int LW = 4;
+    while (LW > 1 && bytes(LW) > 110 * 1024) LW--;
+    const size_t smem = bytes(LW);
     auto k = k_zmask<R, Mask>;
     set_smem(k, smem);
-    k<<<(unsigned)ceil_div(ncols, W), 256, smem, st>>>(zd, ncols, pz, W, ld, mask);
+    k<<<(unsigned)ceil_div(ncols, 1 << LW), kSmemFftThreads, smem, st>>>(zd, ncols, with_magic(pz), LW, mask);
     TTM_LAUNCH_CHECK();
 }
 

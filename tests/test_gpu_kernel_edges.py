@@ -1,0 +1,83 @@
+"""Edge sizes of the kernels' tiles and of the rules that choose between
+kernels, each against the float64 oracle at sampled voxels."""
+import json
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2408_02398_gb300 import synth
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+C_TOL = 2e-5   # FP32 transforms of unit-variance data, as for every correlate test
+W_TOL = 1e-5
+
+
+@pytest.fixture(scope="module")
+def T():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2408_02398_gb300 import build
+    build.build()
+    from paper_2408_02398_gb300 import ttm
+    return ttm
+
+
+@pytest.fixture(scope="module")
+def ctx(T):
+    return T.Context(0)
+
+
+def dev(a, dtype=torch.float32):
+    return torch.as_tensor(np.ascontiguousarray(a), dtype=dtype, device="cuda")
+
+
+def check_correlate(T, ctx, shape, N, r, n, localsum, samples=400, seed=1):
+    V = int(np.prod(shape))
+    tomo = synth.normals(seed, 1, V).reshape(shape).astype(np.float32)
+    tmpl = synth.gaussian_blob_template(N, seed=N)
+    m, _ = O.mask(tmpl.shape, r)
+    field = O.tensor_field(O.normalise_template(tmpl, m)[0], O.rotation_set(4), n)
+    plan = T.Plan(ctx, dev(field, torch.float64), T.params(order_n=n, mask_radius=r, n_rot_base=4), shape)
+    T.ttm_plan_set_localsum(plan, localsum)
+    d_C = torch.empty((field.shape[0],) + tuple(shape), device="cuda")
+    d_w = torch.empty(shape, device="cuda")
+    T.ttm_correlate(plan, dev(tomo), d_C)
+    T.ttm_plan_copy_w(plan, d_w)
+    torch.cuda.synchronize()
+    vox = np.sort(np.random.default_rng(N).choice(V, size=min(V, samples), replace=False))
+    pr = O.Prepared(tomo.astype(np.float64), tmpl, r)
+    w, _, _ = O.local_w(pr.g, pr.m, vox, periodic=True, floor=pr.floor)
+    C = O.correlate(pr.g, field, vox, periodic=True, w=w)
+    assert np.abs(d_w.cpu().numpy().ravel()[vox] - w).max() <= W_TOL * np.abs(w).max()
+    got = d_C.cpu().numpy().reshape(field.shape[0], -1)[:, vox]
+    assert np.abs(got - C).max() <= C_TOL * max(1.0, np.abs(C).max())
+
+
+# shared-memory transforms: line counts that are no multiple of the tile
+# width, every radix, and lengths at which the tile width drops to its least
+@pytest.mark.parametrize("localsum", [0, 1])
+@pytest.mark.parametrize("shape", [(14, 15, 45), (9, 10, 1260), (10, 1120, 9), (1050, 9, 14), (27, 49, 25),
+                                   (16, 24, 40)])
+def test_shared_memory_transform_tiles(T, ctx, shape, localsum):
+    check_correlate(T, ctx, shape, 9, 4.0, 2, localsum)
+
+
+def test_tile_width_of_a_loaded_record(T, tmp_path):
+    """A tuning record may ask for any tile width: it is rounded down to a power of two."""
+    c = T.Context(0)
+    f = tmp_path / "tune.json"
+    T.ttm_autotune_shape(c, (45, 45, 45))
+    T.ttm_autotune_save(c, str(f))
+    text = f.read_text()
+    rec = json.loads(text)
+    rows = rec["lengths"] if isinstance(rec, dict) and "lengths" in rec else rec
+    for row in rows:
+        if not row["reg"]:
+            row["W"] = 12
+    f.write_text("[\n" + ",\n".join(json.dumps(r) for r in rows) + "\n]\n")
+    T.ttm_autotune_load(c, str(f))
+    check_correlate(T, c, (45, 45, 45), 9, 4.0, 2, 0)
