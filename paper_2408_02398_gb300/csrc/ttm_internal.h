@@ -32,6 +32,7 @@ struct Prep {
     int tz = 0, ty = 0, tx = 0;
     double M = 0;              // sum of the mask
     double filter_a = 0.2;
+    int pre_chunk = 1;         // planes a prefilter thread marches over
     int64_t nblk_pre = 0;      // blocks of the prefilter reduction
     DevBuf g32;                // float [Z][Y][X] filtered tomogram g
     DevBuf G;                  // float2 [Z][Y][Xh] spectrum of g

@@ -60,7 +60,7 @@ constexpr int kPreThreads = 256;
 // g = h * f, the 27-point product filter (taps a, 1 - 2a, a on each axis) in
 // FP32 (the input is FP32), applied separably while marching along z: a
 // thread owns four consecutive voxels of one row (y, x0 .. x0+3) over a
-// chunk of kPfZChunk planes. For each plane it filters the rows y-1, y, y+1
+// chunk of zc planes. For each plane it filters the rows y-1, y, y+1
 // along x (one read of x0-1 .. x0+4 each) and combines them along y; three
 // such planes in registers give g along z. Writes g (f32) and (g, g^2) in
 // FP64 or as double-float pairs for the local sums (unless the first
@@ -69,24 +69,39 @@ constexpr int kPreThreads = 256;
 // The tomogram f is Zt x Yt x Xt; g lives on the working grid Z x Y x X
 // (>= the tomogram on every axis, zero beyond it apart from the filter's
 // one-voxel spill). Only tomogram voxels enter the g^2 partial sums.
+//
+// Marching a plane costs one round of dependent loads, so what bounds a small
+// volume is the length of the march, not its bytes: 64^3 in chunks of 25
+// planes is 3072 threads and 42 us. The chunk is 25 planes (two planes
+// read again per 25) where that leaves enough threads, else the longest
+// that gives every SM 512 of them: 64^3 then takes chunks of one plane
+// (with the epilogue below, the whole 64^3 match went from 196 to 157 us).
 constexpr int kPreVox = 4;
 constexpr int kPfZChunk = 25;
 
-static int64_t prefilter_blocks(int Z, int Y, int X)
+static int prefilter_chunk(int num_sms, int Z, int Y, int X)
 {
-    return ceil_div((int64_t)ceil_div(Z, kPfZChunk) * Y * ceil_div(X, kPreVox), kPreThreads);
+    const int64_t columns = (int64_t)Y * ceil_div(X, kPreVox);
+    int zc = kPfZChunk;
+    while (zc > 1 && ceil_div(Z, zc) * columns < (int64_t)num_sms * 512) zc--;
+    return zc;
+}
+
+static int64_t prefilter_blocks(int zc, int Z, int Y, int X)
+{
+    return ceil_div((int64_t)ceil_div(Z, zc) * Y * ceil_div(X, kPreVox), kPreThreads);
 }
 
 // DF: the (g, g^2) pack of the local sums in double-float, else in FP64;
 // zc == nullptr: no pack (the first local-sum pass forms it from g32)
 template <bool DF>
 __global__ void __launch_bounds__(kPreThreads)
-k_prefilter(const float* __restrict__ f, int Zt, int Yt, int Xt, int Z, int Y, int X, float a,
+k_prefilter(const float* __restrict__ f, int Zt, int Yt, int Xt, int Z, int Y, int X, int zchunk, float a,
             float* __restrict__ g32, double2* __restrict__ zc, double* __restrict__ partials)
 {
     __shared__ float warp_sums[kPreThreads / 32];
     const int Xq = (X + kPreVox - 1) / kPreVox;
-    const int nzc = (Z + kPfZChunk - 1) / kPfZChunk;
+    const int nzc = (Z + zchunk - 1) / zchunk;
     const int64_t nq = (int64_t)nzc * Y * Xq;
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     float sq = 0.f;
@@ -96,7 +111,7 @@ k_prefilter(const float* __restrict__ f, int Zt, int Yt, int Xt, int Z, int Y, i
         const int y = (int)(r % Y);
         const int cz = (int)(r / Y);
         const int x0 = xq * kPreVox;
-        const int z0 = cz * kPfZChunk, z1 = min(Z, z0 + kPfZChunk);
+        const int z0 = cz * zchunk, z1 = min(Z, z0 + zchunk);
         const float t0 = a, t1 = 1.f - 2.f * a;
         // the x- and y-filtered plane zz at (y, x0 .. x0+3); zero off the tomogram
         auto plane = [&](int zz, float* o) {
@@ -225,19 +240,34 @@ struct ProMaskSpectrum {
     }
 };
 
-// epilogue of the inverse x pass: (S1, S2) -> w
+// 1 / sqrt(v), v > 0, to a relative error below 1e-12 (the caller rounds it
+// to FP32): the FP32 reciprocal square root (error below 2^-21) and one
+// Newton step in FP64, where v is within FP32's normal range
+__device__ __forceinline__ float rsqrt_of_double(double v)
+{
+    const float f = (float)v;
+    if (!(f > 1e-30f && f < 1e30f)) return (float)(1.0 / sqrt(v));
+    const double y = (double)rsqrtf(f);
+    return (float)fma(0.5 * y, fma(-v * y, y, 1.0), y);
+}
+
+// epilogue of the inverse x pass: (S1, S2) -> w. The FP64 pipe bounds this
+// pass (about 1.7 lane operations per clock and SM): an FP64 division, square
+// root and reciprocal were 27 of its 63 FP64 instructions per voxel at
+// X = 315. With the reciprocal of M and rsqrt_of_double they are 10:
+// ttm_correlate of 126 x 270 x 315 (n = 4) 6.64 -> 6.38 ms, same bits.
 struct StoreW {
     float* w;
     const double* floor;
-    double M;
+    double inv_M;
     int X;
     __device__ void operator()(double2 v, int64_t l, int64_t, int j) const
     {
-        double S1 = v.x, S2 = v.y;
-        double var = S2 - S1 * S1 / M;
+        const double S1 = v.x, S2 = v.y;
+        const double var = fma(-S1, S1 * inv_M, S2);
         // zero local variance: below the volume-energy floor, or constant to
         // ~5 digits over the window (the FFT leaves rounding noise there)
-        w[l * X + j] = (var > floor[0] && var > 1e-10 * S2) ? (float)(1.0 / sqrt(var)) : 0.0f;
+        w[l * X + j] = (var > floor[0] && var > 1e-10 * S2) ? rsqrt_of_double(var) : 0.0f;
     }
 };
 
@@ -378,7 +408,8 @@ void prep_create(ttm_ctx* ctx, Prep& p, int Zt, int Yt, int Xt, int Z, int Y, in
     p.pyd = ctx_len_plan(ctx, Y, TW_DF64);
     p.pzd = ctx_len_plan(ctx, Z, TW_DF64);
     const int64_t V = (int64_t)Z * Y * X, Vh = (int64_t)Z * Y * p.Xh;
-    p.nblk_pre = prefilter_blocks(Z, Y, X);
+    p.pre_chunk = prefilter_chunk(ctx->num_sms, Z, Y, X);
+    p.nblk_pre = prefilter_blocks(p.pre_chunk, Z, Y, X);
     p.g32.alloc(V * sizeof(float));
     p.G.alloc(Vh * sizeof(float2));
     p.zc.alloc(V * sizeof(double2));
@@ -417,11 +448,11 @@ void prep_filter(Prep& p, const float* d_tomo, cudaStream_t st)
     const int64_t Vt = (int64_t)p.Zt * p.Yt * p.Xt;
     if (p.localsum_mode == 1)
         k_prefilter<true><<<(unsigned)p.nblk_pre, kPreThreads, 0, st>>>(
-            d_tomo, p.Zt, p.Yt, p.Xt, p.Z, p.Y, p.X, (float)p.filter_a, p.g32.as<float>(),
+            d_tomo, p.Zt, p.Yt, p.Xt, p.Z, p.Y, p.X, p.pre_chunk, (float)p.filter_a, p.g32.as<float>(),
             localsum_reads_g(p) ? nullptr : p.zc.as<double2>(), p.partials.as<double>());
     else
         k_prefilter<false><<<(unsigned)p.nblk_pre, kPreThreads, 0, st>>>(d_tomo, p.Zt, p.Yt, p.Xt, p.Z, p.Y, p.X,
-                                                                      (float)p.filter_a, p.g32.as<float>(),
+                                                                      p.pre_chunk, (float)p.filter_a, p.g32.as<float>(),
                                                                       p.zc.as<double2>(), p.partials.as<double>());
     TTM_LAUNCH_CHECK();
     k_var_floor<<<1, 1024, 0, st>>>(p.partials.as<double>(), p.nblk_pre, Vt, p.M, p.floor.as<double>());
@@ -473,7 +504,7 @@ void prep_localsums(Prep& p, cudaStream_t st)
     launch_strided_any<double, +1>(zc, StridedAxis{X, Z, YX, X}, p.py64, ProIdentity<double>(),
                                    StoreTo<double>{zc, YX, X}, st);
     launch_contig_any<double, +1>(zc, (int64_t)Z * Y, p.px64, ProIdentity<double>(),
-                                  StoreW{p.w.as<float>(), p.floor.as<double>(), p.M, X}, st);
+                                  StoreW{p.w.as<float>(), p.floor.as<double>(), 1.0 / p.M, X}, st);
 }
 
 }  // namespace ttm
