@@ -5,7 +5,7 @@
 #include <cstring>
 #include <vector>
 
-#include "fft.cuh"
+#include "fft_pfa.cuh"
 
 namespace ttm {
 
@@ -72,6 +72,68 @@ LenPlan with_magic(LenPlan pl)
     return pl;
 }
 
+// the coprime parts of a 7-smooth L, in the order of their rows
+static int pfa_parts(int L, int* g, int* p)
+{
+    int n = 0;
+    for (int r : {2, 3, 5, 7}) {
+        int q = 1;
+        while (L % r == 0) { L /= r; q *= r; }
+        if (q > 1) { g[n] = q; p[n++] = r; }
+    }
+    return n;
+}
+
+void pfa_maps(int L, uint16_t* maps)
+{
+    uint16_t *crt = maps, *rur = maps + L, *kof = maps + 2 * L;
+    int g[4], p[4];
+    const int n = pfa_parts(L, g, p);
+    for (int j = 0; j < L; j++) {
+        int rc = 0, rr = 0, G = 1;
+        for (int i = 0; i < n; i++) {
+            // j = sum (L/g) k_g mod L: k_g = j (L/g)^-1 mod g
+            const int c = (L / g[i]) % g[i];
+            int inv = 0;
+            while ((int64_t)inv * c % g[i] != 1 % g[i]) inv++;
+            rc += G * (j % g[i]);
+            rr += G * (int)((int64_t)j * inv % g[i]);
+            G *= g[i];
+        }
+        crt[j] = (uint16_t)rc;
+        rur[j] = (uint16_t)rr;
+        kof[rr] = (uint16_t)j;
+    }
+}
+
+PfaPlan pfa_plan(const LenPlan& pl)
+{
+    PfaPlan q{};
+    const int L = pl.L;
+    q.L = L;
+    q.tw = reinterpret_cast<const double2*>(pl.tw);
+    q.crt = reinterpret_cast<const uint16_t*>(q.tw + L);
+    q.rur = q.crt + L;
+    q.kof = q.rur + L;
+    auto magic = [](int d) { return d > 1 ? (uint32_t)(((1ull << 32) + d - 1) / d) : 0u; };
+    int g[4], p[4], G = 1;
+    const int n = pfa_parts(L, g, p);
+    for (int i = 0; i < n; i++) {
+        int rest = g[i], Ns = 1;
+        while (rest > 1) {
+            int r = p[i];
+            if (r == 2) r = rest % 8 == 0 ? 8 : (rest % 4 == 0 ? 4 : 2);
+            if (r == 3 && rest % 9 == 0) r = 9;
+            PfaStage& s = q.st[q.nst++];
+            s = PfaStage{r, G, g[i], Ns, g[i] / r, L / (Ns * r), magic(G), magic(g[i] / r), magic(Ns)};
+            Ns *= r;
+            rest /= r;
+        }
+        G *= g[i];
+    }
+    return q;
+}
+
 TwiddleCache::~TwiddleCache()
 {
     for (int i = 0; i < n_; i++) cudaFree(entries_[i].ptr);
@@ -91,11 +153,14 @@ const void* TwiddleCache::get(int L, int kind)
     }
     void* d = nullptr;
     const size_t esz = kind == TW_F32 ? sizeof(float2) : sizeof(double2);
-    const size_t bytes = (size_t)L * esz;
+    // FP64: the three index maps of the prime-factor passes follow the twiddles
+    const size_t maps = kind == TW_F64 ? (3 * (size_t)L * sizeof(uint16_t) + esz - 1) / esz * esz : 0;
+    const size_t bytes = (size_t)L * esz + maps;
     TTM_CUDA_TRY(cudaMalloc(&d, bytes));
     if (kind == TW_F64) {
-        std::vector<double2> h(L);
+        std::vector<double2> h(bytes / sizeof(double2));
         for (int m = 0; m < L; m++) h[m] = make_double2(re[m], im[m]);
+        pfa_maps(L, reinterpret_cast<uint16_t*>(h.data() + L));
         TTM_CUDA_TRY(cudaMemcpy(d, h.data(), bytes, cudaMemcpyHostToDevice));
     } else if (kind == TW_DF64) {
         // (re.hi, re.lo, im.hi, im.lo)

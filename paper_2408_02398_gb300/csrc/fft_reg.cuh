@@ -19,6 +19,7 @@
 
 #include "fft.cuh"
 #include "fft_line3.cuh"
+#include "fft_pfa.cuh"
 
 namespace ttm {
 
@@ -418,15 +419,18 @@ template <typename R, int DIR, class Pro, class Store, typename In = cx<R>>
 inline void launch_strided_any(const In* in, StridedAxis ax, const LenPlan& pl, Pro pro, Store store,
                                cudaStream_t st)
 {
-    if constexpr (std::is_same<R, df64>::value) {
-        if (!pl.no_reg && line3_length(pl.L)) {
-            launch_line3_strided<DIR>(in, ax, pl, pro, store, st);
-            TTM_LAUNCH_CHECK();
-            return;
+    if constexpr (std::is_same<R, double>::value) {
+        launch_pfa_strided<DIR>(in, ax, pl, pro, store, st);
+    } else {
+        if constexpr (std::is_same<R, df64>::value) {
+            if (!pl.no_reg && line3_length(pl.L)) {
+                launch_line3_strided<DIR>(in, ax, pl, pro, store, st);
+                TTM_LAUNCH_CHECK();
+                return;
+            }
         }
-    }
-    int E, P;
-    if (pl.no_reg || !fs_split(pl.L, E, P)) { launch_strided<R, DIR>(in, ax, pl, pro, store, st); return; }
+        int E, P;
+        if (pl.no_reg || !fs_split(pl.L, E, P)) { launch_strided<R, DIR>(in, ax, pl, pro, store, st); return; }
 #define TTM_L(E_, P_)                                                                          \
     {                                                                                          \
         using S = FsShape<R, E_, P_>;                                                          \
@@ -436,24 +440,28 @@ inline void launch_strided_any(const In* in, StridedAxis ax, const LenPlan& pl, 
         TTM_REQUIRE(grid < (1ll << 31), E_SHAPE, "strided pass grid too large");               \
         k<<<(unsigned)grid, S::THREADS, S::SMEM, st>>>(in, ax, pl.tw, pro, store);             \
     }
-    TTM_FS_SWITCH(pl.L, TTM_L)
+        TTM_FS_SWITCH(pl.L, TTM_L)
 #undef TTM_L
-    TTM_LAUNCH_CHECK();
+        TTM_LAUNCH_CHECK();
+    }
 }
 
 template <typename R, int DIR, class Pro, class Store>
 inline void launch_contig_any(const cx<R>* in, int64_t nlines, const LenPlan& pl, Pro pro, Store store,
                               cudaStream_t st)
 {
-    if constexpr (std::is_same<R, df64>::value) {
-        if (!pl.no_reg && line3_length(pl.L)) {
-            launch_line3_contig<DIR>(in, nlines, pl, pro, store, st);
-            TTM_LAUNCH_CHECK();
-            return;
+    if constexpr (std::is_same<R, double>::value) {
+        launch_pfa_contig<DIR>(in, nlines, pl, pro, store, st);
+    } else {
+        if constexpr (std::is_same<R, df64>::value) {
+            if (!pl.no_reg && line3_length(pl.L)) {
+                launch_line3_contig<DIR>(in, nlines, pl, pro, store, st);
+                TTM_LAUNCH_CHECK();
+                return;
+            }
         }
-    }
-    int E, P;
-    if (pl.no_reg || !fs_split(pl.L, E, P)) { launch_contig<R, DIR>(in, nlines, pl, pro, store, st); return; }
+        int E, P;
+        if (pl.no_reg || !fs_split(pl.L, E, P)) { launch_contig<R, DIR>(in, nlines, pl, pro, store, st); return; }
 #define TTM_L(E_, P_)                                                                          \
     {                                                                                          \
         using S = FsShape<R, E_, P_>;                                                          \
@@ -461,9 +469,10 @@ inline void launch_contig_any(const cx<R>* in, int64_t nlines, const LenPlan& pl
         set_smem(k, S::SMEM);                                                                  \
         k<<<(unsigned)ceil_div(nlines, S::W), S::THREADS, S::SMEM, st>>>(in, nlines, pl.tw, pro, store); \
     }
-    TTM_FS_SWITCH(pl.L, TTM_L)
+        TTM_FS_SWITCH(pl.L, TTM_L)
 #undef TTM_L
-    TTM_LAUNCH_CHECK();
+        TTM_LAUNCH_CHECK();
+    }
 }
 
 template <typename R, class Src>

@@ -324,12 +324,12 @@ struct StoreWDF {
     }
 };
 
-// Fused z pass of the local sums: per tile of W adjacent (y, x) columns,
-// the forward transform along z, the product with the (real, even) mask
-// spectrum and the inverse transform, through shared memory (Stockham
-// stages: one copy of each butterfly, which keeps the long FP64 /
-// double-float kernels inside the instruction cache). One read and one
-// write of the (g, g^2) spectrum instead of two each.
+// Fused z pass of the double-float local sums: per tile of W adjacent (y, x)
+// columns, the forward transform along z, the product with the (real, even)
+// mask spectrum and the inverse transform, through shared memory (Stockham
+// stages: one copy of each butterfly, which keeps the long double-float
+// kernel inside the instruction cache). One read and one write of the
+// (g, g^2) spectrum instead of two each. (FP64: k_pfa_zmask.)
 template <typename R, class Mask>
 __global__ void __launch_bounds__(kSmemFftThreads)
 k_zmask(cx<R>* __restrict__ zd, int64_t ncols, LenPlan pl, int LW, Mask mask)
@@ -359,12 +359,10 @@ k_zmask(cx<R>* __restrict__ zd, int64_t ncols, LenPlan pl, int LW, Mask mask)
 template <typename R, class Mask>
 static void launch_zmask(cx<R>* zd, int64_t ncols, const LenPlan& pz, Mask mask, cudaStream_t st)
 {
-    if constexpr (std::is_same<R, df64>::value) {
-        if (!pz.no_reg && line3_length(pz.L)) {
-            launch_line3_zmask(zd, ncols, pz, mask, st);
-            TTM_LAUNCH_CHECK();
-            return;
-        }
+    if (!pz.no_reg && line3_length(pz.L)) {
+        launch_line3_zmask(zd, ncols, pz, mask, st);
+        TTM_LAUNCH_CHECK();
+        return;
     }
     const int Z = pz.L;
     auto bytes = [&](int lw) { return ((2ull << lw) * Z + Z) * sizeof(cx<R>); };
@@ -500,7 +498,7 @@ void prep_localsums(Prep& p, cudaStream_t st)
     launch_contig_any<double, -1>(zc, (int64_t)Z * Y, p.px64, ProIdentity<double>(), StoreTo<double>{zc, X, 1}, st);
     launch_strided_any<double, -1>(zc, StridedAxis{X, Z, YX, X}, p.py64, ProIdentity<double>(),
                                    StoreTo<double>{zc, YX, X}, st);
-    launch_zmask<double>(zc, YX, p.pz64, ProMaskSpectrum{p.mhat.as<double>(), Z, Y, X}, st);
+    launch_pfa_zmask(zc, YX, p.pz64, ProMaskSpectrum{p.mhat.as<double>(), Z, Y, X}, st);
     launch_strided_any<double, +1>(zc, StridedAxis{X, Z, YX, X}, p.py64, ProIdentity<double>(),
                                    StoreTo<double>{zc, YX, X}, st);
     launch_contig_any<double, +1>(zc, (int64_t)Z * Y, p.px64, ProIdentity<double>(),
