@@ -186,7 +186,7 @@ struct ttm_mlp {
     int64_t step = 0;
     ttm::DevBuf params, grad, m, v;
     int64_t cap = 0;  // rows of training scratch
-    ttm::DevBuf xb, ub, a1, h1, a2, h2, y, dy, loss, part;
+    ttm::DevBuf xb, ub, a1, h1, a2, h2, dy, loss, part, gpart;
     ttm::DevBuf image;         // kMlpImageBytes, rebuilt when the parameters change
     bool image_dirty = true;
     bool bf16 = false;         // forward / backward products in BF16 (tensor cores)

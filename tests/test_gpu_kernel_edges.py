@@ -81,3 +81,24 @@ def test_tile_width_of_a_loaded_record(T, tmp_path):
     f.write_text("[\n" + ",\n".join(json.dumps(r) for r in rows) + "\n]\n")
     T.ttm_autotune_load(c, str(f))
     check_correlate(T, c, (45, 45, 45), 9, 4.0, 2, 0)
+
+
+# weight gradients split over the rows: single rows, remainders of the k steps
+# and of the splits, one and two column tiles of W1, and two chunks of rows
+@pytest.mark.parametrize("K,rows", [(6, 1), (15, 63), (28, 65), (28, 4097), (64, 80), (65, 200), (128, 1000),
+                                    (15, 65537)])
+def test_mlp_gradient_splits(T, ctx, K, rows):
+    rng = np.random.default_rng(K + rows)
+    X = rng.standard_normal((rows, K))
+    X /= np.linalg.norm(X, axis=1, keepdims=True)
+    U = rng.standard_normal((rows, 3))
+    U /= np.linalg.norm(U, axis=1, keepdims=True)
+    X, U = X.astype(np.float32), U.astype(np.float32)
+    net = T.Mlp(ctx, K, seed=rows)
+    g = torch.zeros(net.num_params, device="cuda")
+    L = net.loss_grad(dev(X), dev(U), g)
+    _, Lo, go = O.mlp(net.get_params().astype(np.float64), X.astype(np.float64), U.astype(np.float64), want_grad=True)
+    got = g.cpu().numpy()
+    # the bounds of the gradient check in test_gpu_mlp.py
+    assert abs(L - Lo) <= 1e-5 * max(Lo, 1e-3)
+    assert np.abs(got - go).max() <= 1e-4 * np.abs(go).max()
