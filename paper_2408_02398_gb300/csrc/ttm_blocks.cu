@@ -12,50 +12,7 @@
 #include <map>
 #include <vector>
 
-#include "ttm_internal.h"
-
-namespace ttm {
-
-// candidates at z in [cz0, cz1) (and the y, x box), neighbours tested
-// within [nz0, nz1) (and the same y, x box) of a map on a Z x Y x X grid;
-// indices written on the tomogram's grid: ((z + zoff) Yt + y) Xt + x
-__global__ void k_localmax_slab(const float* __restrict__ s, int Y, int X, int cz0, int cz1, int nz0, int nz1,
-                                int y0, int y1, int x0, int x1, int64_t zoff, int Yt, int Xt, int64_t cap,
-                                int64_t* __restrict__ idx, float* __restrict__ val,
-                                unsigned long long* __restrict__ count)
-{
-    const int bx = x1 - x0, by = y1 - y0, bz = cz1 - cz0;
-    const int64_t n = (int64_t)bx * by * bz;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-        const int x = x0 + (int)(t % bx);
-        const int64_t r = t / bx;
-        const int y = y0 + (int)(r % by), z = cz0 + (int)(r / by);
-        const int64_t i = ((int64_t)z * Y + y) * X + x;
-        const float v = s[i];
-        if (!(v == v)) continue;
-        bool is_max = true;
-        for (int dz = -1; dz <= 1 && is_max; dz++)
-            for (int dy = -1; dy <= 1 && is_max; dy++)
-                for (int dx = -1; dx <= 1 && is_max; dx++) {
-                    if (!dz && !dy && !dx) continue;
-                    const int zz = z + dz, yy = y + dy, xx = x + dx;
-                    if (zz < nz0 || zz >= nz1 || yy < y0 || yy >= y1 || xx < x0 || xx >= x1) continue;
-                    const int64_t j = ((int64_t)zz * Y + yy) * X + xx;
-                    const float o = s[j];
-                    // ties go to the lower linear index; the slab's order of
-                    // indices is the tomogram's (same y, x strides per plane)
-                    if (o > v || (o == v && j < i)) is_max = false;
-                }
-        if (!is_max) continue;
-        const unsigned long long pos = atomicAdd(count, 1ull);
-        if ((int64_t)pos < cap) {
-            idx[pos] = (((int64_t)z + zoff) * Yt + y) * Xt + x;
-            val[pos] = v;
-        }
-    }
-}
-
-}  // namespace ttm
+#include "localmax.cuh"
 
 // A block-processing session: the slab table, one plan per distinct slab
 // depth (template spectra on each slab's autotuned working grid), the slab
@@ -106,19 +63,19 @@ extern "C" int ttm_merge_peaks(int64_t n, const int64_t* idx, const float* val, 
     if (n < 0 || P < 0 || min_dist < 0 || Z <= 0 || Y <= 0 || X <= 0 || (n > 0 && (!idx || !val)) ||
         (P > 0 && (!out_idx || !out_val)))
         return -1;
-    std::vector<int64_t> order(n);
-    for (int64_t i = 0; i < n; i++) order[i] = i;
-    std::sort(order.begin(), order.end(), [&](int64_t a, int64_t c) {
-        if (val[a] != val[c]) return val[a] > val[c];
-        return idx[a] < idx[c];
-    });
+    // a heap: only the candidates down to the last accepted one are ordered
+    struct Cand { float v; int64_t i; };
+    auto after = [](const Cand& a, const Cand& b) { return a.v != b.v ? a.v < b.v : a.i > b.i; };
+    std::vector<Cand> c((size_t)n);
+    for (int64_t i = 0; i < n; i++) c[(size_t)i] = Cand{val[i], idx[i]};
+    std::make_heap(c.begin(), c.end(), after);
     const double md2 = min_dist * min_dist;
     std::vector<double> acc;
     int got = 0;
-    for (int64_t o : order) {
-        if (got >= P) break;
-        const int64_t i = idx[o];
-        const double x = (double)(i % X), y = (double)((i / X) % Y), z = (double)(i / ((int64_t)X * Y));
+    for (auto end = c.end(); end != c.begin() && got < P; --end) {
+        std::pop_heap(c.begin(), end, after);
+        const Cand& o = *(end - 1);
+        const double x = (double)(o.i % X), y = (double)((o.i / X) % Y), z = (double)(o.i / ((int64_t)X * Y));
         bool ok = true;
         for (int a = 0; a < got && ok; a++) {
             const double dz = z - acc[3 * a], dy = y - acc[3 * a + 1], dx = x - acc[3 * a + 2];
@@ -126,8 +83,8 @@ extern "C" int ttm_merge_peaks(int64_t n, const int64_t* idx, const float* val, 
         }
         if (!ok) continue;
         acc.push_back(z); acc.push_back(y); acc.push_back(x);
-        out_idx[got] = i;
-        out_val[got] = val[o];
+        out_idx[got] = o.i;
+        out_val[got] = o.v;
         got++;
     }
     return got;
@@ -236,10 +193,11 @@ extern "C" ttm_status ttm_blocked_run(ttm_blocked* B, const float* h_tomo, int m
                               stream);
             if (rc != TTM_OK) throw Error{rc, ttm_last_error(ctx)};
             const Prep& p = plan->prep;
-            k_localmax_slab<<<32 * B->ctx->num_sms, 256, 0, st>>>(B->d_map.as<float>(), p.Y, p.X, o0 - i0, o1 - i0, m0 - i0,
-                                                          m1 - i0, y0, y1, x0, x1, (int64_t)i0, Y, X, B->cap, cidx,
-                                                          cval, B->cnt.as<unsigned long long>());
-            TTM_LAUNCH_CHECK();
+            // ties go to the lower linear index; the slab's order of indices
+            // is the tomogram's (same y, x order per plane)
+            localmax_run(ctx->num_sms, B->d_map.as<float>(),
+                         LmGeom{p.Y, p.X, o0 - i0, o1 - i0, m0 - i0, m1 - i0, y0, y1, x0, x1, (int64_t)i0, Y, X, 0},
+                         B->cap, cidx, cval, B->cnt.as<unsigned long long>(), st);
         }
         unsigned long long n = 0;
         TTM_CUDA_TRY(cudaMemcpyAsync(&n, B->cnt.p, sizeof(n), cudaMemcpyDeviceToHost, st));
