@@ -103,9 +103,10 @@ double make_mask(int tz, int ty, int tx, double r, double soft, std::vector<doub
 // exponents of (w, x, y, z) with sum n (4 per component)
 void rotation_set(int64_t n_base, bool cube, std::vector<double>& q);
 // t' of Eq. 4 (filter, mask, zero mean and unit norm under the mask) of a
-// raw float template, FP64 on the device, returned in tp
+// raw float template, FP64 on the device, returned in tp; d_mask: the mask
+// of the same grid and parameters if it is on the device already
 void normalise_template_dev(ttm_ctx* ctx, const float* d_tmpl, int tz, int ty, int tx, const ttm_field_params& fp,
-                            DevBuf& tp, cudaStream_t st);
+                            DevBuf& tp, cudaStream_t st, const double* d_mask = nullptr);
 void exponents4(int n, std::vector<int>& e);
 // device address of the fixed scratch array of the allocation-free Find
 // Peaks on the current device (looked up once per context)

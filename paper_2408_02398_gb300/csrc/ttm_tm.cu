@@ -14,10 +14,6 @@
 
 namespace ttm {
 
-
-void normalise_template_dev(ttm_ctx* ctx, const float* d_tmpl, int tz, int ty, int tx,
-                            const ttm_field_params& fp, DevBuf& tp, cudaStream_t st);
-
 struct Rot9 { double r[9]; };
 
 __global__ void k_rotate_template(const double* __restrict__ tp, int tz, int ty, int tx, Rot9 R, double scale,

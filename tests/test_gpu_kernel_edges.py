@@ -102,3 +102,76 @@ def test_mlp_gradient_splits(T, ctx, K, rows):
     # the bounds of the gradient check in test_gpu_mlp.py
     assert abs(L - Lo) <= 1e-5 * max(Lo, 1e-3)
     assert np.abs(got - go).max() <= 1e-4 * np.abs(go).max()
+
+
+def brute_peaks(m, box):
+    """Strict 26-neighbour maxima inside the box (ties to the lower index, NaN neither a peak nor a rival)."""
+    z0, z1, y0, y1, x0, x1 = box
+    out = []
+    for z in range(z0, z1):
+        for y in range(y0, y1):
+            for x in range(x0, x1):
+                v = m[z, y, x]
+                if v != v:
+                    continue
+                ok = True
+                for c in range(max(z0, z - 1), min(z1, z + 2)):
+                    for b in range(max(y0, y - 1), min(y1, y + 2)):
+                        for a in range(max(x0, x - 1), min(x1, x + 2)):
+                            o = m[c, b, a]
+                            if o > v or (o == v and (c, b, a) < (z, y, x)):
+                                ok = False
+                if ok:
+                    out.append((-v, (z * m.shape[1] + y) * m.shape[2] + x))
+    return [i for _, i in sorted(out)]
+
+
+# column tiles of 30, rows of 4, chunks of planes; ties, infinities and NaN
+@pytest.mark.parametrize("shape,box", [((19, 9, 70), (0, 19, 0, 9, 0, 70)), ((18, 12, 62), (1, 18, 2, 11, 1, 61)),
+                                       ((5, 7, 31), (0, 5, 0, 7, 0, 31)), ((4, 4, 64), (3, 4, 3, 4, 5, 6)),
+                                       ((33, 5, 33), (0, 33, 0, 5, 2, 32)), ((3, 3, 3), (1, 1, 0, 3, 0, 3))])
+def test_find_peaks_tiles_and_special_values(T, ctx, shape, box):
+    rng = np.random.default_rng(sum(shape))
+    for levels in (3, 1000):
+        m = rng.integers(0, levels, shape).astype(np.float32)
+        m[rng.random(shape) < 0.05] = np.nan
+        m[rng.random(shape) < 0.02] = np.inf
+        m[rng.random(shape) < 0.02] = -np.inf
+        m[0, 0, 0] = -np.inf
+        idx, val = T.ttm_find_peaks_noalloc(ctx, dev(m), box, 16384, 0.0)
+        want = brute_peaks(m, box)
+        assert idx.tolist() == want
+        assert np.array_equal(val, m.ravel()[want])
+
+
+# the reach list (odd and even templates, soft masks) and the path for
+# quaternions that are not unit; peaks at the corners of the valid box
+@pytest.mark.parametrize("scale", [1.0, 1.003])
+@pytest.mark.parametrize("N,r,soft", [(9, 4.0, 0.0), (8, 3.5, 0.0), (12, 3.0, 2.5), (13, 5.0, 1.0)])
+def test_refine_reach_against_direct_sum(T, ctx, N, r, soft, scale):
+    shape = (20, 21, 25)
+    rng = np.random.default_rng(N)
+    tomo = synth.normals(N, 1, int(np.prod(shape))).reshape(shape).astype(np.float32)
+    tmpl = synth.gaussian_blob_template(N, seed=N, std_lo=0.7, std_hi=1.5).astype(np.float32)
+    pr = O.Prepared(tomo.astype(np.float64), tmpl.astype(np.float64), r, soft=soft)
+    field = O.tensor_field(pr.tp, O.rotation_set(1), 2, 4)
+    p = T.params(order_n=2, mask_radius=r, mask_soft_width=soft, dprime=4, n_rot_base=1)
+    plan = T.Plan(ctx, dev(field, torch.float64), p, shape)
+    T.ttm_correlate(plan, dev(tomo), torch.empty((10,) + shape, device="cuda"))
+    d_w = torch.empty(shape, device="cuda")
+    T.ttm_plan_copy_w(plan, d_w)
+    w = d_w.cpu().numpy().astype(np.float64)
+    q = rng.standard_normal((4,) + shape)
+    q = (scale * q / np.linalg.norm(q, axis=0)).astype(np.float32)
+    b = plan.valid_box()
+    at = [(b[0], b[2], b[4]), (b[1] - 1, b[3] - 1, b[5] - 1), (b[0], b[3] - 1, b[4])]
+    peaks = np.array([(z * shape[1] + y) * shape[2] + x for z, y, x in at])
+    idx, quat, lncc = T.ttm_refine_peaks(plan, dev(tmpl), dev(q), peaks, r_s=0.0)
+    assert np.array_equal(idx, peaks)
+    h = N // 2
+    for (z, y, x), ql, c in zip(at, quat, lncc):
+        assert np.array_equal(ql, q[:, z, y, x])
+        tv = synth.resample_rotated(pr.tp, synth.quat_matrix(ql.astype(np.float64)))
+        win = pr.g.reshape(shape)[z - h:z - h + N, y - h:y - h + N, x - h:x - h + N]
+        # FP32 coordinates, samples and partial sums of |t'| = 1 against windows of norm 1 / w
+        assert abs(c - w[z, y, x] * (tv * win).sum()) <= 2e-5
