@@ -163,11 +163,11 @@ const void* TwiddleCache::get(int L, int kind)
         pfa_maps(L, reinterpret_cast<uint16_t*>(h.data() + L));
         TTM_CUDA_TRY(cudaMemcpy(d, h.data(), bytes, cudaMemcpyHostToDevice));
     } else if (kind == TW_DF64) {
-        // (re.hi, re.lo, im.hi, im.lo)
+        // (re.hi, im.hi, re.lo, im.lo)
         std::vector<float4> h(L);
         for (int m = 0; m < L; m++) {
             float rh = (float)re[m], ih = (float)im[m];
-            h[m] = make_float4(rh, (float)(re[m] - (double)rh), ih, (float)(im[m] - (double)ih));
+            h[m] = make_float4(rh, ih, (float)(re[m] - (double)rh), (float)(im[m] - (double)ih));
         }
         TTM_CUDA_TRY(cudaMemcpy(d, h.data(), bytes, cudaMemcpyHostToDevice));
     } else {

@@ -105,12 +105,14 @@ template <int DIR, typename C> __device__ __forceinline__ void dft4(C& a0, C& a1
 // two products instead of a full complex product
 template <int DIR, typename R> __device__ __forceinline__ cx<R> mul_w8_1(cx<R> x, R h)
 {
-    return DIR < 0 ? mk<R>((x.x + x.y) * h, (x.y - x.x) * h) : mk<R>((x.x - x.y) * h, (x.y + x.x) * h);
+    if constexpr (std::is_same<R, df64>::value) return mul_w8_df<DIR>(x, h, false);
+    else return DIR < 0 ? mk<R>((x.x + x.y) * h, (x.y - x.x) * h) : mk<R>((x.x - x.y) * h, (x.y + x.x) * h);
 }
 // x * (-h + DIR h i) = h (-x.x - DIR x.y) + i h (DIR x.x - x.y)
 template <int DIR, typename R> __device__ __forceinline__ cx<R> mul_w8_3(cx<R> x, R h)
 {
-    return DIR < 0 ? mk<R>((x.y - x.x) * h, (-x.x - x.y) * h) : mk<R>((-x.x - x.y) * h, (x.x - x.y) * h);
+    if constexpr (std::is_same<R, df64>::value) return mul_w8_df<DIR>(x, h, true);
+    else return DIR < 0 ? mk<R>((x.y - x.x) * h, (-x.x - x.y) * h) : mk<R>((-x.x - x.y) * h, (x.x - x.y) * h);
 }
 
 template <int DIR, typename R> __device__ __forceinline__ void dft8(cx<R>* v)
@@ -239,7 +241,7 @@ __device__ __forceinline__ void stockham_stage(const cx<R>* __restrict__ in, cx<
             for (int r = 1; r < RAD; r++) {
                 tk += k * step;
                 cx<R> t_ = *tk;
-                if (DIR > 0) t_.y = -t_.y;
+                if (DIR > 0) t_ = cconj(t_);
                 v[r] = cmul(v[r], t_);
             }
         }

@@ -56,9 +56,8 @@ __device__ __forceinline__ void line3_twiddles(dcx* tw, const void* twg)
     for (int i = threadIdx.x; i < S::NTW; i += blockDim.x) {
         const int t = i < S::NTW1 ? (i % S::P) * (i / S::P + 1)
                                   : R1 * ((i - S::NTW1) % R3) * ((i - S::NTW1) / R3 + 1);
-        dcx w = g[t];
-        if (DIR > 0) w.y = -w.y;
-        tw[i] = w;
+        const dcx w = g[t];
+        tw[i] = DIR > 0 ? cconj(w) : w;
     }
 }
 

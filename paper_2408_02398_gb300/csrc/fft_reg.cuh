@@ -33,9 +33,8 @@ __host__ __device__ constexpr int pick_radix(int S)
 template <int DIR, typename R>
 __device__ __forceinline__ cx<R> twid(const cx<R>* __restrict__ tw, int t)
 {
-    cx<R> w = tw[t];
-    if (DIR > 0) w.y = -w.y;
-    return w;
+    const cx<R> w = tw[t];
+    return DIR > 0 ? cconj(w) : w;
 }
 
 // in-place S-point DFT of v (natural order in and out); tw = exp(-2 pi i t / TWL)

@@ -151,7 +151,7 @@ k_prefilter(const float* __restrict__ f, int Zt, int Yt, int Xt, int Z, int Y, i
                     } else if (DF) {
                         // (g, g^2) as double-float pairs; g^2 is exact as hi + lo
                         const df64 s2 = two_prod(g, g);
-                        reinterpret_cast<float4*>(zc)[v0 + k] = make_float4(g, 0.f, s2.hi, s2.lo);
+                        reinterpret_cast<float4*>(zc)[v0 + k] = make_float4(g, s2.hi, 0.f, s2.lo);
                     } else {
                         const double gd = (double)g;
                         zc[v0 + k] = make_double2(gd, gd * gd);
@@ -279,10 +279,7 @@ struct SrcGSquared {
     __device__ dcx operator()(int64_t l, int j) const
     {
         const float v = __ldg(g + l * X + j);
-        dcx r;
-        r.x = df64(v, 0.f);
-        r.y = two_prod(v, v);
-        return r;
+        return make_dcx(df64(v, 0.f), two_prod(v, v));
     }
 };
 
@@ -301,11 +298,7 @@ struct ProMaskSpectrumDF {
         int ay = ky <= Y - ky ? ky : Y - ky;
         int ax = kx <= X - kx ? kx : X - kx;
         const float2 m2 = oct[((int64_t)az * (Y / 2 + 1) + ay) * (X / 2 + 1) + ax];
-        const df64 m(m2.x, m2.y);
-        dcx o;
-        o.x = v.x * m;
-        o.y = v.y * m;
-        return o;
+        return cscale(v, df64(m2.x, m2.y));
     }
 };
 
@@ -316,7 +309,7 @@ struct StoreWDF {
     int X;
     __device__ void operator()(dcx v, int64_t l, int64_t, int j) const
     {
-        const df64 S1 = v.x, S2 = v.y;
+        const df64 S1 = v.x(), S2 = v.y();
         const df64 var = S2 - (S1 * S1) * inv_M;  // the cancellation happens here, in double-float
         const float vf = var.hi + var.lo;
         const bool pos = vf > (float)floor[0] && vf > 1e-10f * (S2.hi + S2.lo);
