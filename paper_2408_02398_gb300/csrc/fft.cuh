@@ -84,19 +84,33 @@ struct OddRadixConst {
 
 // ---------------------------------------------------------- butterflies --
 
+// Sum and difference of two complex values: for FP32 one packed instruction
+// for both parts (a - b as a fused multiply-add by -1, the same rounding),
+// which halves the issue slots of a butterfly's additions.
+template <typename C> __device__ __forceinline__ C padd(C a, C b)
+{
+    if constexpr (std::is_same<C, float2>::value) return __fadd2_rn(a, b);
+    else return cadd(a, b);
+}
+template <typename C> __device__ __forceinline__ C psub(C a, C b)
+{
+    if constexpr (std::is_same<C, float2>::value) return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+    else return csub(a, b);
+}
+
 template <int DIR, typename C> __device__ __forceinline__ void dft2(C* v)
 {
     C a = v[0], b = v[1];
-    v[0] = cadd(a, b);
-    v[1] = csub(a, b);
+    v[0] = padd(a, b);
+    v[1] = psub(a, b);
 }
 
 template <int DIR, typename C> __device__ __forceinline__ void dft4(C& a0, C& a1, C& a2, C& a3)
 {
-    C t0 = cadd(a0, a2), t1 = csub(a0, a2);
-    C t2 = cadd(a1, a3), t3 = cmul_diri<DIR>(csub(a1, a3));
-    a0 = cadd(t0, t2);
-    a2 = csub(t0, t2);
+    C t0 = padd(a0, a2), t1 = psub(a0, a2);
+    C t2 = padd(a1, a3), t3 = cmul_diri<DIR>(psub(a1, a3));
+    a0 = padd(t0, t2);
+    a2 = psub(t0, t2);
     a1 = cadd(t1, t3);
     a3 = csub(t1, t3);
 }
@@ -123,6 +137,18 @@ template <int DIR, typename R> __device__ __forceinline__ void dft8(cx<R>* v)
     dft4<DIR>(o0, o1, o2, o3);
     const R h = (R)OddRadixConst::sqrt_half;
     // w8^1 = h(1 + DIR i), w8^2 = DIR i, w8^3 = h(-1 + DIR i)
+    if constexpr (std::is_same<R, float>::value) {
+        // the products by h are fused into the additions that take them
+        const float2 p = DIR < 0 ? make_float2(o1.x + o1.y, o1.y - o1.x) : make_float2(o1.x - o1.y, o1.y + o1.x);
+        const float2 q = DIR < 0 ? make_float2(o3.y - o3.x, -o3.x - o3.y) : make_float2(-o3.x - o3.y, o3.x - o3.y);
+        const float2 hh = make_float2(h, h), mh = make_float2(-h, -h);
+        const float2 t2 = cmul_diri<DIR>(o2);
+        v[0] = padd(e0, o0); v[4] = psub(e0, o0);
+        v[1] = __ffma2_rn(p, hh, e1); v[5] = __ffma2_rn(p, mh, e1);
+        v[2] = cadd(e2, t2); v[6] = csub(e2, t2);
+        v[3] = __ffma2_rn(q, hh, e3); v[7] = __ffma2_rn(q, mh, e3);
+        return;
+    }
     cx<R> t1 = mul_w8_1<DIR, R>(o1, h);
     cx<R> t2 = cmul_diri<DIR>(o2);
     cx<R> t3 = mul_w8_3<DIR, R>(o3, h);
