@@ -79,9 +79,16 @@ template <typename R> struct FsThreads { static constexpr int value = 256; };
 template <> struct FsThreads<double> { static constexpr int value = 128; };
 template <> struct FsThreads<df64> { static constexpr int value = 128; };
 
+// 128 threads where a thread holds 32 FP32 values (about 100 registers): four or
+// five CTAs per SM in different phases (loading, transforming, storing)
+// instead of two of 256 threads; the x pass of 200 x 512 x 512 (K = 15) went
+// from 1.41 to 1.30 ms, with FP16 spectra on 256 x 512 x 512 (K = 28) from
+// 3.35 to 3.10 ms, the y pass by 0 and 2 %
+template <typename R, int E> constexpr int fs_threads() { return (std::is_same<R, float>::value && E >= 32) ? 128 : FsThreads<R>::value; }
+
 template <typename R, int E, int P> struct FsShape {
     static constexpr int L = E * P;
-    static constexpr int W = FsThreads<R>::value / P;    // lines per CTA
+    static constexpr int W = fs_threads<R, E>() / P;     // lines per CTA
     static constexpr int KS = P + 1;                     // padded stride of k1 in the transpose
     static constexpr int LD = (E * KS) | 1;              // odd line stride
     static constexpr int THREADS = W * P;
@@ -114,7 +121,7 @@ __device__ __forceinline__ void fs_phase1(cx<R>* x, int p, cx<R>* xch, const cx<
 // strided axis: lines (o, i), i adjacent (w fastest in the CTA), elements
 // at o*os + i + j*s. Natural order in and out.
 template <typename R, int E, int P, int DIR, class Pro, class Store, typename In = cx<R>>
-__global__ void __launch_bounds__(FsThreads<R>::value)
+__global__ void __launch_bounds__((fs_threads<R, E>()))
 k_fs_strided(const In* __restrict__ in, StridedAxis ax, const void* twg, Pro pro, Store store)
 {
     using S = FsShape<R, E, P>;
@@ -162,7 +169,7 @@ k_fs_strided(const In* __restrict__ in, StridedAxis ax, const void* twg, Pro pro
 
 // contiguous lines l (elements l*L + j), p fastest in the CTA
 template <typename R, int E, int P, int DIR, class Pro, class Store>
-__global__ void __launch_bounds__(FsThreads<R>::value)
+__global__ void __launch_bounds__((fs_threads<R, E>()))
 k_fs_contig(const cx<R>* __restrict__ in, int64_t nlines, const void* twg, Pro pro, Store store)
 {
     using S = FsShape<R, E, P>;
@@ -207,7 +214,7 @@ k_fs_contig(const cx<R>* __restrict__ in, int64_t nlines, const void* twg, Pro p
 // transform the complex line is staged in natural order (same buffer, after
 // a barrier) for the split into the two half spectra.
 template <typename R, int E, int P, class Src>
-__global__ void __launch_bounds__(FsThreads<R>::value)
+__global__ void __launch_bounds__((fs_threads<R, E>()))
 k_fs_r2c(Src src, int64_t nrows, cx<R>* __restrict__ out, const void* twg)
 {
     using S = FsShape<R, E, P>;
@@ -259,7 +266,7 @@ k_fs_r2c(Src src, int64_t nrows, cx<R>* __restrict__ out, const void* twg)
 // inverse complex-to-real rows (2-for-1, see k_c2r_rows), batched: the
 // component index is the fastest grid index.
 template <typename R, int E, int P, class Sink, typename In = cx<R>>
-__global__ void __launch_bounds__(FsThreads<R>::value)
+__global__ void __launch_bounds__((fs_threads<R, E>()))
 k_fs_c2r(const In* __restrict__ in, int64_t nrows, Sink sink, const void* twg, int nbatch)
 {
     using S = FsShape<R, E, P>;
@@ -314,7 +321,7 @@ k_fs_c2r(const In* __restrict__ in, int64_t nrows, Sink sink, const void* twg, i
 // FP16 / BF16 pairs); gmax (or NULL): the image spectrum is multiplied by
 // 1 / *gmax as it is loaded, so that scaled products stay in FP16 range.
 template <int E, int P, typename TS = float2, typename TW = float2>
-__global__ void __launch_bounds__(FsThreads<float>::value, 2)
+__global__ void __launch_bounds__((fs_threads<float, E>()), 2)
 k_fs_zcorr(const float2* __restrict__ G, const TS* __restrict__ spec, int K, int tzn, int cz, int64_t ncols,
            TW* __restrict__ out, const void* twg, const float* __restrict__ gmax, float oscale)
 {
