@@ -141,10 +141,12 @@ struct ttm_ctx {
     int num_sms = 0;
     ttm::DevBuf probe_tables;  // maximiser probe directions and monomials
     size_t probe_off[5] = {0, 0, 0, 0, 0};
+    int pm_resident[3] = {1, 1, 1};  // CTAs of the plain maximiser (n = 2, 4, 6) per SM
     ttm::DevBuf probe_half;    // FP16 monomial tables for the tensor-core probe product
     size_t probe_half_off[3] = {0, 0, 0};
     ttm::DevBuf probe4;        // quaternion maximiser: probe quaternions and FP16 monomials
-    size_t probe4_off[4] = {0, 0, 0, 0};
+    size_t probe4_off[5] = {0, 0, 0, 0, 0};
+    int p4_resident[3] = {1, 1, 1};  // CTAs of the quaternion maximiser (n = 2, 4, 6) per SM
     void* peak_scratch = nullptr;  // device address of the allocation-free Find Peaks scratch
     // sticky record of an expired bounded device wait (int, device) and the
     // poll limit of such waits

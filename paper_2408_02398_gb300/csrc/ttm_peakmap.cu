@@ -239,6 +239,7 @@ struct ProbeTables {
     const float* phi4;
     const float* phi6;
     const uint4* far;          // [kProbes] 128-bit rows: probes j with |d_i . d_j| < cos(kStartSepDeg)
+    const uint4* far_cells;    // the same with rows and bits in the order 8 cell + member
     // FP16 copies [kProbes][pm_kxs(n)] (components beyond K and the row
     // padding zero) for the tensor-core probe product
     const __half* phi2h;
@@ -313,6 +314,7 @@ k_peakmap(const float* __restrict__ C, int64_t V, float* __restrict__ score, flo
     constexpr int KXS = pm_kxs(N);
     constexpr int kStarts = nstarts(N);
     __shared__ float4 sdir[kProbes];
+    __shared__ uint4 sfar[kProbes];
     // xs / keys: the staged input, then the cell keys (see pm_key_at);
     // phih: [kProbes][KXS] FP16 weighted monomials
     extern __shared__ __align__(16) __half pm_smem[];
@@ -324,7 +326,7 @@ k_peakmap(const float* __restrict__ C, int64_t V, float* __restrict__ score, flo
         const uint4* src = reinterpret_cast<const uint4*>(ph);
         uint4* dst = reinterpret_cast<uint4*>(phih);
         for (int i = threadIdx.x; i < kProbes * KXS / 8; i += blockDim.x) dst[i] = src[i];
-        for (int i = threadIdx.x; i < kProbes; i += blockDim.x) sdir[i] = tabs.dir[i];
+        for (int i = threadIdx.x; i < kProbes; i += blockDim.x) { sdir[i] = tabs.dir[i]; sfar[i] = tabs.far_cells[i]; }
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -441,57 +443,48 @@ k_peakmap(const float* __restrict__ C, int64_t V, float* __restrict__ score, flo
             }
             // Starts by angular suppression over the cell bests: the best probe,
             // then the best cell best farther than kStartSepDeg from every start
-            // taken and within kStartMargin ||C||_F of the best. The first pass
-            // keeps the cells within the margin (an integer compare of keys) and
-            // farther than kStartSepDeg from the best; each later pass, over the
-            // kept cells only, drops those near the newest start.
+            // taken and within kStartMargin ||C||_F of the best. The 16 keys are
+            // read once, each used with 15 - cell below it, so that one maximum
+            // carries key and cell (the lowest cell of equal keys); whether a
+            // cell's best is far from the starts is one bit of the starts' rows
+            // of the far table (bit 8 cell + member), combined with AND. Against
+            // direction dot products and a loop over the cells left, lane by
+            // lane, and with the grid of plain_run: 9.93 -> 8.54 ms on 200 x 512
+            // x 512 (n = 4), 1.53 -> 1.33 ms on 64 x 256 x 256 (n = 6), the same
+            // maps bit for bit.
             int sj[kStarts];
             bool live[kStarts];
             {
+                uint32_t kw[kCells / 2];
+    #pragma unroll
+                for (int r = 0; r < kCells / 2; r++) kw[r] = xs[r * kPvStride + threadIdx.x];
+                auto key = [&](int cl) {
+                    return ((cl & 1) ? kw[cl / 2] & 0xFFFF0000u : kw[cl / 2] << 16) | (uint32_t)(kCells - 1 - cl);
+                };
                 uint32_t best = 0u;
-                int bc = 0;
     #pragma unroll
-                for (int cl = 0; cl < kCells; cl++) {
-                    const uint32_t kk = keys[pm_key_at(cl, threadIdx.x)];
-                    if (kk > best) { best = kk; bc = cl; }
-                }
-                sj[0] = cell_row(bc, best & 7u);
-                live[0] = true;
+                for (int cl = 0; cl < kCells; cl++) best = max(best, key(cl));
+                uint32_t fw[4] = {~0u, ~0u, ~0u, ~0u};
+                uint32_t pick = best;
+                // (a zero key, that of no number, is never a further start)
+                const uint32_t thr = max(pm_hkey(pm_hkey_value(best >> 16) - kStartMargin, 0u) << 16, 0x10000u);
     #pragma unroll
-                for (int s = 1; s < kStarts; s++) { sj[s] = sj[0]; live[s] = false; }
-                const uint32_t thr = pm_hkey(pm_hkey_value(best) - kStartMargin, 0u);
-                uint32_t alive = 0u, bk = 0u;
-                int bcell = -1;
-                {
-                    const float4 ds = sdir[sj[0]];
+                for (int s = 0; s < kStarts; s++) {
+                    const int cell = kCells - 1 - (int)(pick & 15u);
+                    const uint32_t mem = (pick >> 16) & 7u;
+                    live[s] = pick != 0u;
+                    sj[s] = cell_row(cell, mem);
+                    if (s + 1 == kStarts) break;
+                    const uint4 f = sfar[8 * cell + mem];
+                    fw[0] &= f.x; fw[1] &= f.y; fw[2] &= f.z; fw[3] &= f.w;
+                    pick = 0u;
     #pragma unroll
                     for (int cl = 0; cl < kCells; cl++) {
-                        const uint32_t kk = keys[pm_key_at(cl, threadIdx.x)];
-                        if (kk < thr) continue;
-                        const float4 dj = sdir[cell_row(cl, kk & 7u)];
-                        if (fabsf(dj.x * ds.x + dj.y * ds.y + dj.z * ds.z) < kStartSepCos) {
-                            alive |= 1u << cl;
-                            if (kk > bk) { bk = kk; bcell = cl; }
-                        }
+                        const uint32_t k = key(cl);
+                        const uint32_t far = (fw[cl >> 2] >> ((k >> 16) & 7u)) & (1u << (8 * (cl & 3)));
+                        if (k >= thr && far) pick = max(pick, k);
                     }
-                }
-    #pragma unroll
-                for (int s = 1; s < kStarts; s++) {
-                    if (bcell < 0) break;
-                    sj[s] = cell_row(bcell, bk & 7u);
-                    live[s] = true;
-                    alive &= ~(1u << bcell);
-                    if (s + 1 == kStarts) break;
-                    const float4 ds = sdir[sj[s]];
-                    bk = 0u;
-                    bcell = -1;
-                    for (uint32_t m = alive; m; m &= m - 1) {
-                        const int cl = __ffs((int)m) - 1;
-                        const uint32_t kk = keys[pm_key_at(cl, threadIdx.x)];
-                        const float4 dj = sdir[cell_row(cl, kk & 7u)];
-                        if (fabsf(dj.x * ds.x + dj.y * ds.y + dj.z * ds.z) >= kStartSepCos) alive &= ~(1u << cl);
-                        else if (kk > bk) { bk = kk; bcell = cl; }
-                    }
+                    if (!live[s]) pick = 0u;
                 }
             }
             __syncwarp();  // the key rows are restaged by the next voxel block
@@ -871,6 +864,15 @@ void build_probe_tables(std::vector<float>& out, size_t off[5])
             const double dot = std::fabs(d[3 * i] * d[3 * j] + d[3 * i + 1] * d[3 * j + 1] + d[3 * i + 2] * d[3 * j + 2]);
             if (dot < cmax) far[i * 4 + j / 32] |= 1u << (j % 32);
         }
+    // the same in the order 8 cell + member. No two probes have |d . d'| within
+    // 6e-5 of the limit, so FP32 and FP64 products agree on every pair.
+    std::vector<uint32_t> fc(kProbes * 4, 0u);
+    for (int i = 0; i < kProbes; i++)
+        for (int j = 0; j < kProbes; j++) {
+            const int ri = cell_row(i >> 3, i & 7), rj = cell_row(j >> 3, j & 7);
+            if (far[ri * 4 + rj / 32] >> (rj % 32) & 1u) fc[i * 4 + j / 32] |= 1u << (j % 32);
+        }
+    far.insert(far.end(), fc.begin(), fc.end());
     out.resize(out.size() + far.size(), 0.f);
     std::memcpy(&out[off[4]], far.data(), far.size() * sizeof(uint32_t));
 }
@@ -884,8 +886,21 @@ __global__ void k_phi_half(const float* __restrict__ phi, int KP, int K, int KXS
     }
 }
 
+// declares the dynamic shared memory of k_peakmap<N> on the current device and
+// returns the CTAs of it that an SM holds
+template <int N> static int pm_residency()
+{
+    TTM_CUDA_TRY(cudaFuncSetAttribute(k_peakmap<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pm_smem_bytes(N)));
+    int ctas = 0;
+    TTM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, k_peakmap<N>, kPmThreads, pm_smem_bytes(N)));
+    return std::max(1, ctas);
+}
+
 void upload_probe_tables(ttm_ctx* ctx)
 {
+    ctx->pm_resident[0] = pm_residency<2>();
+    ctx->pm_resident[1] = pm_residency<4>();
+    ctx->pm_resident[2] = pm_residency<6>();
     std::vector<float> h;
     size_t off[5];
     build_probe_tables(h, off);
@@ -915,6 +930,7 @@ static ProbeTables probe_tables(ttm_ctx* ctx)
     return ProbeTables{reinterpret_cast<const float4*>(base + ctx->probe_off[0]), base + ctx->probe_off[1],
                        base + ctx->probe_off[2], base + ctx->probe_off[3],
                        reinterpret_cast<const uint4*>(base + ctx->probe_off[4]),
+                       reinterpret_cast<const uint4*>(base + ctx->probe_off[4]) + kProbes,
                        hb + ctx->probe_half_off[0], hb + ctx->probe_half_off[1], hb + ctx->probe_half_off[2]};
 }
 
@@ -926,12 +942,13 @@ static void plain_run(ttm_ctx* ctx, int n, const float* C, int64_t V, float* sco
     const int64_t items = geo.mode == PM_BOX ? (int64_t)geo.bz * geo.by * geo.bx : V;
     const int64_t blocks = std::max<int64_t>(1, ceil_div(items, kPmThreads));
     const size_t smem = pm_smem_bytes(n);
-    // enough CTAs to fill every SM several times, then a grid stride
-    const int64_t grid = std::min<int64_t>(blocks, (int64_t)ctx->num_sms * 32);
-    // static tables + dynamic probe values can exceed the default 48 KB
-    // total, so the dynamic size is always declared
+    // 16 whole waves of resident CTAs, each with a grid stride. Newton work
+    // differs between regions of a volume, so one wave ends unevenly (10.0 ms
+    // on 200 x 512 x 512; 2, 4, 8, 16, 32, 64 waves: 9.49, 9.11, 8.95, 8.87,
+    // 8.86, 8.93; one block per CTA 9.46), and a part of a wave idles SMs: the
+    // former 32 CTAs per SM were 4.6 waves of 7, or at n = 6 6.4 waves of 5.
+    const int64_t grid = std::min<int64_t>(blocks, (int64_t)ctx->num_sms * ctx->pm_resident[n / 2 - 1] * 16);
 #define TTM_PM_LAUNCH(N_)                                                                          \
-    TTM_CUDA_TRY(cudaFuncSetAttribute(k_peakmap<N_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
     k_peakmap<N_><<<(unsigned)grid, kPmThreads, smem, st>>>(C, V, score, orient, frob, t, geo);
     switch (n) {
         case 2: TTM_PM_LAUNCH(2); break;
