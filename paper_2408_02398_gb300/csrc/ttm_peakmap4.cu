@@ -20,7 +20,7 @@
 //    bits), in shared memory [cell][thread];
 //  * starts by angular suppression over the cell bests: the best probe,
 //    then the best cell best farther than 25 degrees (|q . q_s| <
-//    cos 25 deg) from every start taken, if within 0.2 ||C||_F (n = 4) or
+//    cos 25 deg, one bit of a table) from every start taken, if within 0.2 ||C||_F (n = 4) or
 //    0.5 ||C||_F (n = 6) of the best, up to 4 (n = 4) or 6 (n = 6) starts;
 //  * n = 2 needs no probes: p = q^T A q with A_ij = C_{e_i + e_j}, whose
 //    maximum over unit q is the top eigenpair of the symmetric 4 x 4
@@ -318,6 +318,9 @@ struct Probe4Tables {
     const __half* phi2h;  // [kP4][p4_kxs(2)] FP16 weighted monomials
     const __half* phi4h;  // [kP4][p4_kxs(4)]
     const __half* phi6h;  // [kP4][p4_kxs(6)]
+    // [kP4] rows of kP4 bits, both in the order 8 cell + member: the second
+    // probe (rounded to FP16) is farther than 25 degrees from the first
+    const uint4* far;
 };
 
 // Top eigenpair of the symmetric 4 x 4 matrix A (00 01 02 03 11 12 13 22
@@ -402,7 +405,7 @@ __device__ __forceinline__ int key_at(int c, int col) { return 2 * ((c >> 1) * k
 template <int N>
 __host__ __device__ constexpr size_t p4_smem_bytes()
 {
-    return p4_key_bytes(N) + sizeof(float4) * kP4 + sizeof(__half) * (size_t)kP4 * p4_kxs(N) + sizeof(uint2) * kP4;
+    return p4_key_bytes(N) + sizeof(float4) * kP4 + sizeof(__half) * (size_t)kP4 * p4_kxs(N);
 }
 
 template <int N>
@@ -420,18 +423,11 @@ k_peakmap4(const float* __restrict__ C, int64_t V, float* __restrict__ score, fl
     uint32_t* xs = reinterpret_cast<uint32_t*>(p4_smem);  // staged input (aliases the keys)
     float4* sdir = reinterpret_cast<float4*>(p4_smem + p4_key_bytes(N));
     __half* phih = reinterpret_cast<__half*>(sdir + kP4);
-    // FP16 copies of the directions, only for the 25-degree separation tests
-    uint2* sdirh = reinterpret_cast<uint2*>(phih + kP4 * KXS);
     {
         const uint4* src = reinterpret_cast<const uint4*>(N == 2 ? tabs.phi2h : (N == 4 ? tabs.phi4h : tabs.phi6h));
         uint4* dst = reinterpret_cast<uint4*>(phih);
         for (int i = threadIdx.x; i < kP4 * KXS / 8; i += blockDim.x) dst[i] = src[i];
-        for (int i = threadIdx.x; i < kP4; i += blockDim.x) {
-            const float4 d = tabs.dir[i];
-            sdir[i] = d;
-            const __half2 a = __floats2half2_rn(d.x, d.y), b = __floats2half2_rn(d.z, d.w);
-            sdirh[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
-        }
+        for (int i = threadIdx.x; i < kP4; i += blockDim.x) sdir[i] = tabs.dir[i];
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -534,64 +530,60 @@ k_peakmap4(const float* __restrict__ C, int64_t V, float* __restrict__ score, fl
             }
             __syncwarp();
         }
-        // starts: the best probe, then by angular suppression over the cell
-        // bests: the first pass keeps the cells within 0.2 ||C||_F of the
-        // best (an integer compare of keys) that lie farther than 25 degrees
-        // from it; each later start is the best kept cell, and the next pass
-        // (over the kept cells only) drops those within 25 degrees of it.
-        // Start rows are packed 9 bits each.
+        // Starts: the best probe, then by angular suppression over the cell
+        // bests the best one within the margin (an integer compare of keys)
+        // that lies farther than 25 degrees from every start taken. The 64
+        // keys are read two to a word, each used with 63 - cell below it, so that one
+        // maximum carries key and cell (the lowest cell of equal keys);
+        // whether a cell's best is far from the starts is one bit of the
+        // starts' rows of the far table, combined with AND. Against direction
+        // dot products and a loop over the cells left, lane by lane:
+        // 6.17 -> 5.86 ms on 100 x 256 x 256 (n = 4), the same maps. Start
+        // rows are packed 9 bits each.
         uint64_t rows = 0;
-        int ns = 1;
+        int ns = 0;
         {
-            uint32_t best = 0u;
-            int bc = 0;
-#pragma unroll 8
-            for (int cl = 0; cl < kP4Cells; cl++) {
-                const uint32_t kk = keys[key_at(cl, threadIdx.x)];
-                if (kk > best) { best = kk; bc = cl; }
+            // (the key words are read again for every start: 32 of them do not fit
+            // beside the components)
+            const volatile uint32_t* kp = xs + threadIdx.x;
+            uint32_t fw[kP4 / 32];
+#pragma unroll
+            for (int r = 0; r < kP4 / 32; r++) fw[r] = ~0u;
+            auto key = [](uint32_t kw, int cl) {
+                return ((cl & 1) ? kw & 0xFFFF0000u : kw << 16) | (uint32_t)(kP4Cells - 1 - cl);
+            };
+            uint32_t pick = 0u;
+#pragma unroll
+            for (int r = 0; r < kP4Cells / 2; r++) {
+                const uint32_t kw = kp[r * kXStride];
+                pick = max(pick, max(key(kw, 2 * r), key(kw, 2 * r + 1)));
             }
-            int last = p4_row(bc, best & 7u);
-            rows = (uint64_t)last;
-            const uint32_t thr = hkey(hkey_value(best) - p4_margin(N), 0u);
-            uint64_t alive = 0ull;
-            uint32_t bk = 0u;
-            int bcell = -1;
-            {
-                const float4 ds = sdir[last];
-#pragma unroll 4
-                for (int cl = 0; cl < kP4Cells; cl++) {
-                    const uint32_t kk = keys[key_at(cl, threadIdx.x)];
-                    if (kk < thr) continue;
-                    const uint2 dh = sdirh[p4_row(cl, kk & 7u)];
-                    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&dh.x));
-                    const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&dh.y));
-                    const float dt = fabsf(a.x * ds.x + a.y * ds.y + b.x * ds.z + b.y * ds.w);
-                    if (dt < kP4SepCos) {
-                        alive |= 1ull << cl;
-                        if (kk > bk) { bk = kk; bcell = cl; }
+            // (a zero key, that of no number, is never a further start)
+            const uint32_t thr = max(hkey(hkey_value(pick >> 16) - p4_margin(N), 0u) << 16, 0x10000u);
+#pragma unroll 1
+            for (;;) {
+                const int cell = kP4Cells - 1 - (int)(pick & 63u);
+                const uint32_t mem = (pick >> 16) & 7u;
+                rows |= (uint64_t)p4_row(cell, mem) << (9 * ns);
+                if (++ns == kStarts) break;
+                const uint4* f = tabs.far + (8 * cell + mem) * (kP4 / 128);
+#pragma unroll
+                for (int r = 0; r < kP4 / 128; r++) {
+                    const uint4 v4 = __ldg(f + r);
+                    fw[4 * r] &= v4.x; fw[4 * r + 1] &= v4.y; fw[4 * r + 2] &= v4.z; fw[4 * r + 3] &= v4.w;
+                }
+                pick = 0u;
+#pragma unroll
+                for (int r = 0; r < kP4Cells / 2; r++) {
+                    const uint32_t kw = kp[r * kXStride];
+#pragma unroll
+                    for (int cl = 2 * r; cl <= 2 * r + 1; cl++) {
+                        const uint32_t k = key(kw, cl);
+                        const uint32_t far = (fw[cl >> 2] >> ((k >> 16) & 7u)) & (1u << (8 * (cl & 3)));
+                        if (k >= thr && far) pick = max(pick, k);
                     }
                 }
-            }
-#pragma unroll 1
-            for (int s = 1; s < kStarts && bcell >= 0; s++) {
-                last = p4_row(bcell, bk & 7u);
-                rows |= (uint64_t)last << (9 * s);
-                ns = s + 1;
-                alive &= ~(1ull << bcell);
-                if (s + 1 == kStarts) break;
-                const float4 ds = sdir[last];
-                bk = 0u;
-                bcell = -1;
-                for (uint64_t m = alive; m; m &= m - 1) {
-                    const int cl = __ffsll((long long)m) - 1;
-                    const uint32_t kk = keys[key_at(cl, threadIdx.x)];
-                    const uint2 dh = sdirh[p4_row(cl, kk & 7u)];
-                    const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&dh.x));
-                    const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&dh.y));
-                    const float dt = fabsf(a.x * ds.x + a.y * ds.y + b.x * ds.z + b.y * ds.w);
-                    if (dt >= kP4SepCos) alive &= ~(1ull << cl);
-                    else if (kk > bk) { bk = kk; bcell = cl; }
-                }
+                if (!pick) break;
             }
         }
         __syncwarp();  // the key rows are restaged by the next voxel block
@@ -703,8 +695,42 @@ __global__ void k_phi4_half(const float* __restrict__ phi, int KP, int K, int KX
     }
 }
 
+// one word of the far table per thread: row i, probes 32 w .. 32 w + 31, in the
+// order 8 cell + member. The second probe's direction is rounded to FP16, as
+// the selection always took it (the nearest pair is 3e-6 from the limit,
+// so the order of the FP32 sum does not matter).
+__global__ void k_far4(const float4* __restrict__ dir, uint32_t* __restrict__ out)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= kP4 * kP4 / 32) return;
+    const int i = t / (kP4 / 32), w = t % (kP4 / 32);
+    const float4 ds = dir[p4_row(i >> 3, i & 7)];
+    uint32_t bits = 0u;
+    for (int k = 0; k < 32; k++) {
+        const int j = 32 * w + k;
+        const float4 d = dir[p4_row(j >> 3, j & 7)];
+        const float2 a = __half22float2(__floats2half2_rn(d.x, d.y)), b = __half22float2(__floats2half2_rn(d.z, d.w));
+        const float dt = fabsf(a.x * ds.x + a.y * ds.y + b.x * ds.z + b.y * ds.w);
+        if (dt < kP4SepCos) bits |= 1u << k;
+    }
+    out[t] = bits;
+}
+
+// declares the dynamic shared memory of k_peakmap4<N> on the current device
+// and returns the CTAs of it that an SM holds
+template <int N> static int p4_residency()
+{
+    TTM_CUDA_TRY(cudaFuncSetAttribute(k_peakmap4<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p4_smem_bytes<N>()));
+    int ctas = 0;
+    TTM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, k_peakmap4<N>, kP4Threads, p4_smem_bytes<N>()));
+    return std::max(1, ctas);
+}
+
 void upload_probe_tables4(ttm_ctx* ctx)
 {
+    ctx->p4_resident[0] = p4_residency<2>();
+    ctx->p4_resident[1] = p4_residency<4>();
+    ctx->p4_resident[2] = p4_residency<6>();
     std::vector<float> h;
     size_t off[4];
     build_probe4(h, off);
@@ -714,7 +740,8 @@ void upload_probe_tables4(ttm_ctx* ctx)
     const size_t dir_bytes = sizeof(float4) * kP4;
     const size_t h2 = sizeof(__half) * (size_t)kP4 * p4_kxs(2), h4 = sizeof(__half) * (size_t)kP4 * p4_kxs(4);
     const size_t h6 = sizeof(__half) * (size_t)kP4 * p4_kxs(6);
-    ctx->probe4.alloc(dir_bytes + h2 + h4 + h6);
+    const size_t far_bytes = (size_t)kP4 * kP4 / 8;
+    ctx->probe4.alloc(dir_bytes + h2 + h4 + h6 + far_bytes);
     TTM_CUDA_TRY(cudaMemcpy(ctx->probe4.p, f32.p, dir_bytes, cudaMemcpyDeviceToDevice));
     unsigned char* base = ctx->probe4.as<unsigned char>();
     k_phi4_half<<<64, 256>>>(f32.as<float>() + off[1], p4_kp(2), ncomp4(2), p4_kxs(2),
@@ -726,7 +753,12 @@ void upload_probe_tables4(ttm_ctx* ctx)
     k_phi4_half<<<64, 256>>>(f32.as<float>() + off[3], p4_kp(6), ncomp4(6), p4_kxs(6),
                              reinterpret_cast<__half*>(base + dir_bytes + h2 + h4));
     TTM_LAUNCH_CHECK();
+    static_assert((sizeof(__half) * kP4) % 16 == 0, "the far table starts on a 16-byte boundary");
+    k_far4<<<kP4 * kP4 / 32 / 256, 256>>>(reinterpret_cast<const float4*>(base),
+                                          reinterpret_cast<uint32_t*>(base + dir_bytes + h2 + h4 + h6));
+    TTM_LAUNCH_CHECK();
     TTM_CUDA_TRY(cudaDeviceSynchronize());
+    ctx->probe4_off[4] = dir_bytes + h2 + h4 + h6;
     ctx->probe4_off[0] = 0;
     ctx->probe4_off[1] = dir_bytes;
     ctx->probe4_off[2] = dir_bytes + h2;
@@ -740,15 +772,16 @@ void peakmap4_run(ttm_ctx* ctx, int n, const float* C, int64_t V, float* score, 
     const Probe4Tables t{reinterpret_cast<const float4*>(base + ctx->probe4_off[0]),
                          reinterpret_cast<const __half*>(base + ctx->probe4_off[1]),
                          reinterpret_cast<const __half*>(base + ctx->probe4_off[2]),
-                         reinterpret_cast<const __half*>(base + ctx->probe4_off[3])};
+                         reinterpret_cast<const __half*>(base + ctx->probe4_off[3]),
+                         reinterpret_cast<const uint4*>(base + ctx->probe4_off[4])};
     const int64_t blocks = std::max<int64_t>(1, ceil_div(V, kP4Threads));
-    // two resident CTAs per SM (one at n = 6); a grid stride balances the
-    // uneven Newton work
-    const int64_t grid = std::min<int64_t>(blocks, (int64_t)ctx->num_sms * 16);
+    // whole waves of resident CTAs (two per SM, one at n = 6), each with a grid
+    // stride: several, as the Newton work is uneven, but few, as a CTA copies
+    // up to 103 KB of tables first
+    const int64_t grid = std::min<int64_t>(blocks, (int64_t)ctx->num_sms * ctx->p4_resident[n / 2 - 1] * 8);
 #define TTM_P4_LAUNCH(N_)                                                                                       \
     {                                                                                                            \
         const size_t smem = p4_smem_bytes<N_>();                                                                 \
-        TTM_CUDA_TRY(cudaFuncSetAttribute(k_peakmap4<N_>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
         k_peakmap4<N_><<<(unsigned)grid, kP4Threads, smem, st>>>(C, V, score, orient, frob, t);                 \
     }
     switch (n) {
