@@ -146,7 +146,6 @@ struct ttm_ctx {
     size_t probe_half_off[3] = {0, 0, 0};
     ttm::DevBuf probe4;        // quaternion maximiser: probe quaternions and FP16 monomials
     size_t probe4_off[5] = {0, 0, 0, 0, 0};
-    int p4_resident[3] = {1, 1, 1};  // CTAs of the quaternion maximiser (n = 2, 4, 6) per SM
     void* peak_scratch = nullptr;  // device address of the allocation-free Find Peaks scratch
     // sticky record of an expired bounded device wait (int, device) and the
     // poll limit of such waits

@@ -258,6 +258,7 @@ __host__ __device__ constexpr int pm_kxs(int n) { return pm_kx(n) + 8; }
 __host__ __device__ constexpr int pm_rows(int n) { return pm_kx(n) / 2 > kCells / 2 ? pm_kx(n) / 2 : kCells / 2; }
 __host__ __device__ constexpr size_t pm_smem_bytes(int n)
 {
+    if (n == 2) return 0;  // no probes: the closed form
     return sizeof(uint32_t) * (size_t)pm_rows(n) * kPvStride + sizeof(__half) * (size_t)kProbes * pm_kxs(n);
 }
 // a probe value with the member index m (0..7) in its low 3 mantissa bits:
@@ -321,8 +322,8 @@ k_peakmap(const float* __restrict__ C, int64_t V, float* __restrict__ score, flo
     uint32_t* xs = reinterpret_cast<uint32_t*>(pm_smem);
     uint16_t* keys = reinterpret_cast<uint16_t*>(pm_smem);
     __half* phih = pm_smem + 2 * pm_rows(N) * kPvStride;
-    {
-        const __half* ph = N == 2 ? tabs.phi2h : (N == 4 ? tabs.phi4h : tabs.phi6h);
+    if constexpr (N > 2) {
+        const __half* ph = N == 4 ? tabs.phi4h : tabs.phi6h;
         const uint4* src = reinterpret_cast<const uint4*>(ph);
         uint4* dst = reinterpret_cast<uint4*>(phih);
         for (int i = threadIdx.x; i < kProbes * KXS / 8; i += blockDim.x) dst[i] = src[i];

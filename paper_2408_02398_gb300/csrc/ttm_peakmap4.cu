@@ -405,6 +405,7 @@ __device__ __forceinline__ int key_at(int c, int col) { return 2 * ((c >> 1) * k
 template <int N>
 __host__ __device__ constexpr size_t p4_smem_bytes()
 {
+    if (N == 2) return 0;  // no probes: the closed form
     return p4_key_bytes(N) + sizeof(float4) * kP4 + sizeof(__half) * (size_t)kP4 * p4_kxs(N);
 }
 
@@ -423,8 +424,8 @@ k_peakmap4(const float* __restrict__ C, int64_t V, float* __restrict__ score, fl
     uint32_t* xs = reinterpret_cast<uint32_t*>(p4_smem);  // staged input (aliases the keys)
     float4* sdir = reinterpret_cast<float4*>(p4_smem + p4_key_bytes(N));
     __half* phih = reinterpret_cast<__half*>(sdir + kP4);
-    {
-        const uint4* src = reinterpret_cast<const uint4*>(N == 2 ? tabs.phi2h : (N == 4 ? tabs.phi4h : tabs.phi6h));
+    if constexpr (N > 2) {
+        const uint4* src = reinterpret_cast<const uint4*>(N == 4 ? tabs.phi4h : tabs.phi6h);
         uint4* dst = reinterpret_cast<uint4*>(phih);
         for (int i = threadIdx.x; i < kP4 * KXS / 8; i += blockDim.x) dst[i] = src[i];
         for (int i = threadIdx.x; i < kP4; i += blockDim.x) sdir[i] = tabs.dir[i];
@@ -716,21 +717,10 @@ __global__ void k_far4(const float4* __restrict__ dir, uint32_t* __restrict__ ou
     out[t] = bits;
 }
 
-// declares the dynamic shared memory of k_peakmap4<N> on the current device
-// and returns the CTAs of it that an SM holds
-template <int N> static int p4_residency()
-{
-    TTM_CUDA_TRY(cudaFuncSetAttribute(k_peakmap4<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p4_smem_bytes<N>()));
-    int ctas = 0;
-    TTM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, k_peakmap4<N>, kP4Threads, p4_smem_bytes<N>()));
-    return std::max(1, ctas);
-}
-
 void upload_probe_tables4(ttm_ctx* ctx)
 {
-    ctx->p4_resident[0] = p4_residency<2>();
-    ctx->p4_resident[1] = p4_residency<4>();
-    ctx->p4_resident[2] = p4_residency<6>();
+    TTM_CUDA_TRY(cudaFuncSetAttribute(k_peakmap4<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p4_smem_bytes<4>()));
+    TTM_CUDA_TRY(cudaFuncSetAttribute(k_peakmap4<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p4_smem_bytes<6>()));
     std::vector<float> h;
     size_t off[4];
     build_probe4(h, off);
@@ -775,10 +765,13 @@ void peakmap4_run(ttm_ctx* ctx, int n, const float* C, int64_t V, float* score, 
                          reinterpret_cast<const __half*>(base + ctx->probe4_off[3]),
                          reinterpret_cast<const uint4*>(base + ctx->probe4_off[4])};
     const int64_t blocks = std::max<int64_t>(1, ceil_div(V, kP4Threads));
-    // whole waves of resident CTAs (two per SM, one at n = 6), each with a grid
-    // stride: several, as the Newton work is uneven, but few, as a CTA copies
-    // up to 103 KB of tables first
-    const int64_t grid = std::min<int64_t>(blocks, (int64_t)ctx->num_sms * ctx->p4_resident[n / 2 - 1] * 8);
+    // One voxel block per CTA (a grid stride beyond the grid's limit): the
+    // Newton work of a block varies so much that a CTA of ten ends long after
+    // its neighbours, and the SM waits for it with the slots of its other warps
+    // empty. 100 x 256 x 256, n = 4, in 8, 16, 32, 64 waves, one block per CTA:
+    // 6.05, 5.76, 4.92, 4.29, 4.29 ms; 64 x 128 x 256, n = 6: 6.88, 5.29, 4.19,
+    // 4.30, 4.29 ms. The 66 (101) KB of tables that each CTA copies come from L2.
+    const int64_t grid = std::min<int64_t>(blocks, (int64_t)1 << 30);
 #define TTM_P4_LAUNCH(N_)                                                                                       \
     {                                                                                                            \
         const size_t smem = p4_smem_bytes<N_>();                                                                 \
