@@ -105,6 +105,9 @@ ttm_plan::~ttm_plan()
     std::sort(free_ev.begin(), free_ev.end());
     free_ev.erase(std::unique(free_ev.begin(), free_ev.end()), free_ev.end());
     for (cudaEvent_t e : free_ev) cudaEventDestroy(e);
+    if (forked) cudaEventDestroy(forked);
+    if (joined) cudaEventDestroy(joined);
+    if (side) cudaStreamDestroy(side);
 }
 
 static const char* kStageNames[ST_COUNT] = {"prefilter", "image_spectrum", "local_sums", "zpass_fused",

@@ -290,9 +290,59 @@ void plan_build_spectra(ttm_plan* P, const double* d_field)
     TTM_CUDA_TRY(cudaStreamSynchronize(st));
 }
 
+// The local sums of one ttm_correlate, forked to the plan's side stream and
+// joined before the x pass, whose epilogue reads w.
+//
+// In FP64 they are bound by the FP64 pipe and issue an instruction in one of
+// five slots; the image spectrum and the z and y passes are FP32 work that
+// fits beside them where the CTAs of both find room: a 64^3 match 155 -> 133
+// us, ttm_correlate 126 x 270 x 315 (n = 4) 5.56 -> 5.39 ms. (FP64 passes
+// confined to a part of each SM by persistent CTAs left more room, 5.0 ms, but
+// are slower by themselves, and the 64^3 match with them: 148 us.) In
+// double-float both sides want the same FP32 pipes (8.11 against 8.09 ms on
+// 200 x 512 x 512), so they run in sequence, as they do while the stages are
+// timed.
+struct SideSums {
+    ttm_plan* P;
+    cudaStream_t st;
+    bool open = false;
+    SideSums(ttm_plan* P_, cudaStream_t st_) : P(P_), st(st_)
+    {
+        if (P->prep.localsum_mode != TTM_LOCALSUM_FP64 || P->timing) {
+            prep_localsums(P->prep, st);
+            stage_end(P, ST_LOCALSUM, st);
+            return;
+        }
+        TTM_CUDA_TRY(cudaEventRecord(P->forked, st));
+        TTM_CUDA_TRY(cudaStreamWaitEvent(P->side, P->forked, 0));
+        open = true;
+        try {
+            prep_localsums(P->prep, P->side);
+        } catch (...) {
+            end();
+            throw;
+        }
+    }
+    // `st` waits for the sums
+    void join()
+    {
+        if (!open) return;
+        open = false;
+        TTM_CUDA_TRY(cudaEventRecord(P->joined, P->side));
+        TTM_CUDA_TRY(cudaStreamWaitEvent(st, P->joined, 0));
+    }
+    void end() noexcept
+    {
+        if (!open) return;
+        open = false;
+        if (cudaEventRecord(P->joined, P->side) == cudaSuccess) cudaStreamWaitEvent(st, P->joined, 0);
+    }
+    ~SideSums() { end(); }
+};
+
 // z, y and x passes with 16-bit spectra and work buffer (FP32 arithmetic)
 template <typename T16>
-static void correlate_passes16(ttm_plan* P, float* d_C, cudaStream_t st)
+static void correlate_passes16(ttm_plan* P, float* d_C, SideSums& sums, cudaStream_t st)
 {
     Prep& p = P->prep;
     const int Z = p.Z, Y = p.Y, X = p.X, Xh = p.Xh;
@@ -311,6 +361,7 @@ static void correlate_passes16(ttm_plan* P, float* d_C, cudaStream_t st)
     launch_strided_any<float, +1>(work, StridedAxis{Xh, (int64_t)P->K * Z, ncols, Xh}, p.py32, ProIdentity<float>(),
                                   StoreTo16<T16>{work, ncols, Xh, P->work_q}, st);
     stage_end(P, ST_YPASS, st);
+    sums.join();
     launch_c2r_any<float>(work, (int64_t)Z * Y,
                           SinkNormaliseScaled{d_C, p.w.as<float>(), P->spec_scale.as<float>(), gmax, V, X}, p.px32,
                           P->K, st);
@@ -326,19 +377,15 @@ void correlate_run(ttm_plan* P, const float* d_tomo, float* d_C, cudaStream_t st
     stage_begin(P, st);
     prep_filter(p, d_tomo, st);
     stage_end(P, ST_FILTER, st);
-    // (the local sums were measured running on a second stream beside the
-    // spectrum and the z/y passes: both slowed down by as much as they
-    // overlapped, so they run in sequence)
-    prep_localsums(p, st);
-    stage_end(P, ST_LOCALSUM, st);
+    SideSums sums(P, st);
     prep_spectrum(p, st);
     stage_end(P, ST_SPECTRUM, st);
     if (P->prec == TTM_PREC_FP16_SPECTRA) {
-        correlate_passes16<__half2>(P, d_C, st);
+        correlate_passes16<__half2>(P, d_C, sums, st);
         return;
     }
     if (P->prec == TTM_PREC_BF16_SPECTRA) {
-        correlate_passes16<__nv_bfloat162>(P, d_C, st);
+        correlate_passes16<__nv_bfloat162>(P, d_C, sums, st);
         return;
     }
     float2* work = P->work.as<float2>();
@@ -349,6 +396,7 @@ void correlate_run(ttm_plan* P, const float* d_tomo, float* d_C, cudaStream_t st
     launch_strided_any<float, +1>(work, StridedAxis{Xh, (int64_t)P->K * Z, ncols, Xh}, p.py32, ProIdentity<float>(),
                                   StoreTo<float>{work, ncols, Xh}, st);
     stage_end(P, ST_YPASS, st);
+    sums.join();
     launch_c2r_any<float>(work, (int64_t)Z * Y, SinkNormalise{d_C, p.w.as<float>(), V, X}, p.px32, P->K, st);
     stage_end(P, ST_XPASS, st);
 }
@@ -417,6 +465,9 @@ extern "C" ttm_status ttm_plan_create_padded(ttm_ctx* ctx, const double* d_field
         P->cand_count.alloc(sizeof(unsigned long long));
         P->fb_count.alloc(sizeof(unsigned long long));
         TTM_CUDA_TRY(cudaMemset(P->fb_count.p, 0, sizeof(unsigned long long)));
+        TTM_CUDA_TRY(cudaStreamCreateWithFlags(&P->side, cudaStreamNonBlocking));
+        TTM_CUDA_TRY(cudaEventCreateWithFlags(&P->forked, cudaEventDisableTiming));
+        TTM_CUDA_TRY(cudaEventCreateWithFlags(&P->joined, cudaEventDisableTiming));
         *out = P;
         return TTM_OK;
     } catch (const Error& e) {

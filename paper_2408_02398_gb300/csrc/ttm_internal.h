@@ -170,6 +170,10 @@ struct ttm_plan {
     ttm::DevBuf cand_count;  // unsigned long long [1]
     ttm::DevBuf fb_count;    // unsigned long long [1]: learned-maximiser fallbacks of the last call
     int64_t cand_cap = 0;
+    // FP64 local sums beside the image spectrum and the z and y passes: their
+    // stream and the events that fork and join it (see correlate_run)
+    cudaStream_t side = nullptr;
+    cudaEvent_t forked = nullptr, joined = nullptr;
     // stage timing
     bool timing = false;
     cudaEvent_t open_ev = nullptr;

@@ -175,3 +175,40 @@ def test_refine_reach_against_direct_sum(T, ctx, N, r, soft, scale):
         win = pr.g.reshape(shape)[z - h:z - h + N, y - h:y - h + N, x - h:x - h + N]
         # FP32 coordinates, samples and partial sums of |t'| = 1 against windows of norm 1 / w
         assert abs(c - w[z, y, x] * (tv * win).sum()) <= 2e-5
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_side_stream_local_sums_on_user_streams(T, ctx, prec):
+    """FP64 local sums run beside the FP32 passes: the same bits on any stream, back to back, and replayed from a graph."""
+    shape, N, r = (24, 21, 20), 7, 3.0
+    tmpl = synth.gaussian_blob_template(N, seed=N)
+    m, _ = O.mask(tmpl.shape, r)
+    field = dev(O.tensor_field(O.normalise_template(tmpl, m)[0], O.rotation_set(4), 2), torch.float64)
+    tomos = [dev(synth.normals(k, 1, int(np.prod(shape))).reshape(shape)) for k in (1, 2, 3)]
+    plan = T.Plan(ctx, field, T.params(order_n=2, mask_radius=r, n_rot_base=4), shape, precision=prec)
+    T.ttm_plan_enable_timing(plan, True)  # timed stages run in sequence
+    want = []
+    for t in tomos:
+        d_C = torch.empty((6,) + shape, device="cuda")
+        T.ttm_correlate(plan, t, d_C)
+        want.append(d_C)
+    torch.cuda.synchronize()
+    T.ttm_plan_enable_timing(plan, False)
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    got = [torch.empty((6,) + shape, device="cuda") for _ in tomos]
+    with torch.cuda.stream(s):
+        for t, c in zip(tomos, got):
+            T.ttm_correlate(plan, t, c)
+    s.synchronize()
+    for a, b in zip(want, got):
+        assert torch.equal(a, b)
+    d_C, d_t = torch.zeros((6,) + shape, device="cuda"), tomos[0].clone()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        T.ttm_correlate(plan, d_t, d_C)
+    for t, w in zip(tomos, want):
+        d_t.copy_(t)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(d_C, w)
