@@ -89,15 +89,15 @@ void pfa_maps(int L, uint16_t* maps)
     uint16_t *crt = maps, *rur = maps + L, *kof = maps + 2 * L;
     int g[4], p[4];
     const int n = pfa_parts(L, g, p);
+    int inv[4] = {0, 0, 0, 0};  // (L/g)^-1 mod g
+    for (int i = 0; i < n; i++)
+        while ((int64_t)inv[i] * (L / g[i]) % g[i] != 1 % g[i]) inv[i]++;
     for (int j = 0; j < L; j++) {
         int rc = 0, rr = 0, G = 1;
         for (int i = 0; i < n; i++) {
             // j = sum (L/g) k_g mod L: k_g = j (L/g)^-1 mod g
-            const int c = (L / g[i]) % g[i];
-            int inv = 0;
-            while ((int64_t)inv * c % g[i] != 1 % g[i]) inv++;
             rc += G * (j % g[i]);
-            rr += G * (int)((int64_t)j * inv % g[i]);
+            rr += G * (int)((int64_t)j * inv[i] % g[i]);
             G *= g[i];
         }
         crt[j] = (uint16_t)rc;
