@@ -188,6 +188,9 @@ void ttm_plan_valid_box(const ttm_plan* plan, int* box6);
  * g(x+.)^2, summed in FP64; w = 0 where the local variance is zero to
  * rounding: at most 1e-8 * M * mean(g^2) (a window too empty for the FP32
  * correlation to resolve) or at most 1e-10 * S2.
+ * With FP64 local sums part of the work runs on a stream that the plan owns,
+ * forked from `stream` and joined to it by events within the call (also under
+ * stream capture). Calls on one plan share its workspace and must not overlap.
  *   d_tomo  float32 [Z][Y][X] (device)
  *   d_C     float32 [K][Z][Y][X] output (device) */
 ttm_status ttm_correlate(ttm_plan* plan, const float* d_tomo, float* d_C, void* stream);
