@@ -79,16 +79,30 @@ template <typename R> struct FsThreads { static constexpr int value = 256; };
 template <> struct FsThreads<double> { static constexpr int value = 128; };
 template <> struct FsThreads<df64> { static constexpr int value = 128; };
 
-// 128 threads where a thread holds 32 FP32 values (about 100 registers): four or
-// five CTAs per SM in different phases (loading, transforming, storing)
-// instead of two of 256 threads; the x pass of 200 x 512 x 512 (K = 15) went
-// from 1.41 to 1.30 ms, with FP16 spectra on 256 x 512 x 512 (K = 28) from
-// 3.35 to 3.10 ms, the y pass by 0 and 2 %
-template <typename R, int E> constexpr int fs_threads() { return (std::is_same<R, float>::value && E >= 32) ? 128 : FsThreads<R>::value; }
+// Half the threads where a thread holds 32 FP32 values (about 100 registers):
+// four or five CTAs per SM in different phases (loading, transforming,
+// storing) instead of two of 256 threads. Row passes (contiguous lines): x
+// pass of 200 x 512 x 512 (K = 15) 1.41 -> 1.30 ms, with FP16 spectra on
+// 256 x 512 x 512 (K = 28) 3.35 -> 3.10 ms.
+template <typename R, int E, int P> constexpr int fs_threads() { return (std::is_same<R, float>::value && E >= 32) ? 128 : FsThreads<R>::value; }
+// The strided passes only while a CTA keeps 8 adjacent lines: at 1024 (P =
+// 32) 128 threads are 4 lines, and the y pass of 32 x 1024 x 1024 (K = 15)
+// takes 1.69 ms so against 0.94 (FP16 spectra 1.24 against 0.74).
+template <typename R, int E, int P> constexpr int fs_threads_strided() { return P <= 16 ? fs_threads<R, E, P>() : FsThreads<R>::value; }
+// The fused z pass, which reads each spectrum once and holds more in
+// registers, while a row of its tile fills a 32-byte sector of the stored
+// spectra: 1024 x 256 x 128 (K = 15) FP32 1.77 ms with 128 threads, 1.79
+// with 256; FP16 1.82 against 1.67; at 512 128 threads win in both (0.62
+// against 0.74, 0.59 against 0.67 on 512 x 128 x 256).
+template <int E, int P, typename TS> constexpr int fs_threads_z()
+{
+    constexpr int T = fs_threads<float, E, P>();
+    return T / P * sizeof(TS) >= 32 ? T : FsThreads<float>::value;
+}
 
-template <typename R, int E, int P> struct FsShape {
+template <typename R, int E, int P, int T = fs_threads<R, E, P>()> struct FsShape {
     static constexpr int L = E * P;
-    static constexpr int W = fs_threads<R, E>() / P;     // lines per CTA
+    static constexpr int W = T / P;                      // lines per CTA
     static constexpr int KS = P + 1;                     // padded stride of k1 in the transpose
     static constexpr int LD = (E * KS) | 1;              // odd line stride
     static constexpr int THREADS = W * P;
@@ -121,10 +135,11 @@ __device__ __forceinline__ void fs_phase1(cx<R>* x, int p, cx<R>* xch, const cx<
 // strided axis: lines (o, i), i adjacent (w fastest in the CTA), elements
 // at o*os + i + j*s. Natural order in and out.
 template <typename R, int E, int P, int DIR, class Pro, class Store, typename In = cx<R>>
-__global__ void __launch_bounds__((fs_threads<R, E>()))
+__global__ void __launch_bounds__((fs_threads_strided<R, E, P>()))
 k_fs_strided(const In* __restrict__ in, StridedAxis ax, const void* twg, Pro pro, Store store)
 {
-    using S = FsShape<R, E, P>;
+    using S = FsShape<R, E, P, fs_threads_strided<R, E, P>()>;
+    static_assert(!std::is_same<R, float>::value || S::W >= 8, "a strided tile of fewer than 8 lines");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<R>* tw = reinterpret_cast<cx<R>*>(smem_raw);
     cx<R>* xa = tw + S::L;
@@ -169,7 +184,7 @@ k_fs_strided(const In* __restrict__ in, StridedAxis ax, const void* twg, Pro pro
 
 // contiguous lines l (elements l*L + j), p fastest in the CTA
 template <typename R, int E, int P, int DIR, class Pro, class Store>
-__global__ void __launch_bounds__((fs_threads<R, E>()))
+__global__ void __launch_bounds__((fs_threads<R, E, P>()))
 k_fs_contig(const cx<R>* __restrict__ in, int64_t nlines, const void* twg, Pro pro, Store store)
 {
     using S = FsShape<R, E, P>;
@@ -214,7 +229,7 @@ k_fs_contig(const cx<R>* __restrict__ in, int64_t nlines, const void* twg, Pro p
 // transform the complex line is staged in natural order (same buffer, after
 // a barrier) for the split into the two half spectra.
 template <typename R, int E, int P, class Src>
-__global__ void __launch_bounds__((fs_threads<R, E>()))
+__global__ void __launch_bounds__((fs_threads<R, E, P>()))
 k_fs_r2c(Src src, int64_t nrows, cx<R>* __restrict__ out, const void* twg)
 {
     using S = FsShape<R, E, P>;
@@ -266,7 +281,7 @@ k_fs_r2c(Src src, int64_t nrows, cx<R>* __restrict__ out, const void* twg)
 // inverse complex-to-real rows (2-for-1, see k_c2r_rows), batched: the
 // component index is the fastest grid index.
 template <typename R, int E, int P, class Sink, typename In = cx<R>>
-__global__ void __launch_bounds__((fs_threads<R, E>()))
+__global__ void __launch_bounds__((fs_threads<R, E, P>()))
 k_fs_c2r(const In* __restrict__ in, int64_t nrows, Sink sink, const void* twg, int nbatch)
 {
     using S = FsShape<R, E, P>;
@@ -321,11 +336,12 @@ k_fs_c2r(const In* __restrict__ in, int64_t nrows, Sink sink, const void* twg, i
 // FP16 / BF16 pairs); gmax (or NULL): the image spectrum is multiplied by
 // 1 / *gmax as it is loaded, so that scaled products stay in FP16 range.
 template <int E, int P, typename TS = float2, typename TW = float2>
-__global__ void __launch_bounds__((fs_threads<float, E>()), 2)
+__global__ void __launch_bounds__((fs_threads_z<E, P, TS>()), 2)
 k_fs_zcorr(const float2* __restrict__ G, const TS* __restrict__ spec, int K, int tzn, int cz, int64_t ncols,
            TW* __restrict__ out, const void* twg, const float* __restrict__ gmax, float oscale)
 {
-    using S = FsShape<float, E, P>;
+    using S = FsShape<float, E, P, fs_threads_z<E, P, TS>()>;
+    static_assert(S::W * sizeof(TS) >= 32, "a row of the tile is less than a sector of the spectra");
     constexpr int Z = S::L;
     constexpr int ZG = Z | 1;  // odd row stride of the image-spectrum tile
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -439,7 +455,7 @@ inline void launch_strided_any(const In* in, StridedAxis ax, const LenPlan& pl, 
         if (pl.no_reg || !fs_split(pl.L, E, P)) { launch_strided<R, DIR>(in, ax, pl, pro, store, st); return; }
 #define TTM_L(E_, P_)                                                                          \
     {                                                                                          \
-        using S = FsShape<R, E_, P_>;                                                          \
+        using S = FsShape<R, E_, P_, fs_threads_strided<R, E_, P_>()>;                         \
         auto k = k_fs_strided<R, E_, P_, DIR, Pro, Store, In>;                                   \
         set_smem(k, S::SMEM);                                                                  \
         int64_t grid = ax.outer * ceil_div(ax.inner, S::W);                                    \
@@ -506,7 +522,7 @@ inline bool launch_zcorr_fs(const float2* G, const TS* spec, int K, int tzn, int
     if (pz.no_reg || !fs_split(pz.L, E, P)) return false;
 #define TTM_L(E_, P_)                                                                          \
     {                                                                                          \
-        using S = FsShape<float, E_, P_>;                                                      \
+        using S = FsShape<float, E_, P_, fs_threads_z<E_, P_, TS>()>;                          \
         const size_t smem = S::SMEM + (size_t)S::W * (S::L | 1) * sizeof(float2);              \
         auto k = k_fs_zcorr<E_, P_, TS, TW>;                                                   \
         set_smem(k, smem);                                                                     \
