@@ -86,31 +86,34 @@ struct OddRadixConst {
 
 // Sum and difference of two complex values: for FP32 one packed instruction
 // for both parts (a - b as a fused multiply-add by -1, the same rounding),
-// which halves the issue slots of a butterfly's additions.
-template <typename C> __device__ __forceinline__ C padd(C a, C b)
+// which halves the issue slots of a butterfly's additions. PK = false takes
+// the scalar instructions, the same results: operands have to lie in aligned
+// register pairs, and where a pass forms its values part by part the moves
+// into pairs can cost more (fs_c2r_packed).
+template <bool PK, typename C> __device__ __forceinline__ C padd(C a, C b)
 {
-    if constexpr (std::is_same<C, float2>::value) return __fadd2_rn(a, b);
+    if constexpr (PK && std::is_same<C, float2>::value) return __fadd2_rn(a, b);
     else return cadd(a, b);
 }
-template <typename C> __device__ __forceinline__ C psub(C a, C b)
+template <bool PK, typename C> __device__ __forceinline__ C psub(C a, C b)
 {
-    if constexpr (std::is_same<C, float2>::value) return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
+    if constexpr (PK && std::is_same<C, float2>::value) return __ffma2_rn(b, make_float2(-1.f, -1.f), a);
     else return csub(a, b);
 }
 
-template <int DIR, typename C> __device__ __forceinline__ void dft2(C* v)
+template <int DIR, bool PK = true, typename C> __device__ __forceinline__ void dft2(C* v)
 {
     C a = v[0], b = v[1];
-    v[0] = padd(a, b);
-    v[1] = psub(a, b);
+    v[0] = padd<PK>(a, b);
+    v[1] = psub<PK>(a, b);
 }
 
-template <int DIR, typename C> __device__ __forceinline__ void dft4(C& a0, C& a1, C& a2, C& a3)
+template <int DIR, bool PK = true, typename C> __device__ __forceinline__ void dft4(C& a0, C& a1, C& a2, C& a3)
 {
-    C t0 = padd(a0, a2), t1 = psub(a0, a2);
-    C t2 = padd(a1, a3), t3 = cmul_diri<DIR>(psub(a1, a3));
-    a0 = padd(t0, t2);
-    a2 = psub(t0, t2);
+    C t0 = padd<PK>(a0, a2), t1 = psub<PK>(a0, a2);
+    C t2 = padd<PK>(a1, a3), t3 = cmul_diri<DIR>(psub<PK>(a1, a3));
+    a0 = padd<PK>(t0, t2);
+    a2 = psub<PK>(t0, t2);
     a1 = cadd(t1, t3);
     a3 = csub(t1, t3);
 }
@@ -129,21 +132,21 @@ template <int DIR, typename R> __device__ __forceinline__ cx<R> mul_w8_3(cx<R> x
     else return DIR < 0 ? mk<R>((x.y - x.x) * h, (-x.x - x.y) * h) : mk<R>((-x.x - x.y) * h, (x.x - x.y) * h);
 }
 
-template <int DIR, typename R> __device__ __forceinline__ void dft8(cx<R>* v)
+template <int DIR, typename R, bool PK = true> __device__ __forceinline__ void dft8(cx<R>* v)
 {
     cx<R> e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
     cx<R> o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
-    dft4<DIR>(e0, e1, e2, e3);
-    dft4<DIR>(o0, o1, o2, o3);
+    dft4<DIR, PK>(e0, e1, e2, e3);
+    dft4<DIR, PK>(o0, o1, o2, o3);
     const R h = (R)OddRadixConst::sqrt_half;
     // w8^1 = h(1 + DIR i), w8^2 = DIR i, w8^3 = h(-1 + DIR i)
-    if constexpr (std::is_same<R, float>::value) {
+    if constexpr (PK && std::is_same<R, float>::value) {
         // the products by h are fused into the additions that take them
         const float2 p = DIR < 0 ? make_float2(o1.x + o1.y, o1.y - o1.x) : make_float2(o1.x - o1.y, o1.y + o1.x);
         const float2 q = DIR < 0 ? make_float2(o3.y - o3.x, -o3.x - o3.y) : make_float2(-o3.x - o3.y, o3.x - o3.y);
         const float2 hh = make_float2(h, h), mh = make_float2(-h, -h);
         const float2 t2 = cmul_diri<DIR>(o2);
-        v[0] = padd(e0, o0); v[4] = psub(e0, o0);
+        v[0] = padd<PK>(e0, o0); v[4] = psub<PK>(e0, o0);
         v[1] = __ffma2_rn(p, hh, e1); v[5] = __ffma2_rn(p, mh, e1);
         v[2] = cadd(e2, t2); v[6] = csub(e2, t2);
         v[3] = __ffma2_rn(q, hh, e3); v[7] = __ffma2_rn(q, mh, e3);
@@ -226,14 +229,14 @@ template <int DIR, typename R> __device__ __forceinline__ void dft7(cx<R>* v)
     v[4] = pm_diri<DIR, R>(A3, B3, false);
 }
 
-template <int RAD, int DIR, typename R> __device__ __forceinline__ void dft(cx<R>* v)
+template <int RAD, int DIR, typename R, bool PK = true> __device__ __forceinline__ void dft(cx<R>* v)
 {
-    if constexpr (RAD == 2) dft2<DIR>(v);
+    if constexpr (RAD == 2) dft2<DIR, PK>(v);
     else if constexpr (RAD == 3) dft3<DIR, R>(v);
-    else if constexpr (RAD == 4) dft4<DIR>(v[0], v[1], v[2], v[3]);
+    else if constexpr (RAD == 4) dft4<DIR, PK>(v[0], v[1], v[2], v[3]);
     else if constexpr (RAD == 5) dft5<DIR, R>(v);
     else if constexpr (RAD == 7) dft7<DIR, R>(v);
-    else dft8<DIR, R>(v);
+    else dft8<DIR, R, PK>(v);
     // double-float butterflies add without renormalising (df64.cuh): once
     // per output here
     if constexpr (std::is_same<R, df64>::value) {

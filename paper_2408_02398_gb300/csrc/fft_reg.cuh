@@ -37,14 +37,15 @@ __device__ __forceinline__ cx<R> twid(const cx<R>* __restrict__ tw, int t)
     return DIR > 0 ? cconj(w) : w;
 }
 
-// in-place S-point DFT of v (natural order in and out); tw = exp(-2 pi i t / TWL)
-template <int S, int DIR, int TWL, typename R>
+// in-place S-point DFT of v (natural order in and out); tw = exp(-2 pi i t / TWL);
+// PK: packed FP32 additions (padd in fft.cuh)
+template <int S, int DIR, int TWL, typename R, bool PK = true>
 __device__ __forceinline__ void dft_reg(cx<R>* v, const cx<R>* __restrict__ tw)
 {
     if constexpr (S == 1) {
         return;
     } else if constexpr (is_base_radix(S)) {
-        dft<S, DIR, R>(v);
+        dft<S, DIR, R, PK>(v);
     } else {
         constexpr int S1 = pick_radix(S);
         constexpr int S2 = S / S1;
@@ -55,7 +56,7 @@ __device__ __forceinline__ void dft_reg(cx<R>* v, const cx<R>* __restrict__ tw)
             cx<R> t[S2];
 #pragma unroll
             for (int m = 0; m < S2; m++) t[m] = v[p1 + S1 * m];
-            dft_reg<S2, DIR, TWL, R>(t, tw);
+            dft_reg<S2, DIR, TWL, R, PK>(t, tw);
 #pragma unroll
             for (int k1 = 0; k1 < S2; k1++) {
                 if (p1 * k1 != 0) t[k1] = cmul(t[k1], twid<DIR, R>(tw, p1 * k1 * (TWL / S)));
@@ -67,7 +68,7 @@ __device__ __forceinline__ void dft_reg(cx<R>* v, const cx<R>* __restrict__ tw)
             cx<R> u[S1];
 #pragma unroll
             for (int p1 = 0; p1 < S1; p1++) u[p1] = T[p1][k1];
-            dft<S1, DIR, R>(u);
+            dft<S1, DIR, R, PK>(u);
 #pragma unroll
             for (int k2 = 0; k2 < S1; k2++) v[k1 + S2 * k2] = u[k2];
         }
@@ -119,11 +120,11 @@ __device__ __forceinline__ void fs_load_tw(cx<R>* tw, const void* g, int L)
 
 // phase 1 of the forward four-step: E-point DFT + twiddles, then the
 // transposed write xch[k1 * KS + p] (xch = this line's buffer)
-template <typename R, int E, int P, int DIR>
+template <typename R, int E, int P, int DIR, bool PK = true>
 __device__ __forceinline__ void fs_phase1(cx<R>* x, int p, cx<R>* xch, const cx<R>* tw)
 {
     using S = FsShape<R, E, P>;
-    dft_reg<E, DIR, S::L, R>(x, tw);
+    dft_reg<E, DIR, S::L, R, PK>(x, tw);
 #pragma unroll
     for (int k1 = 1; k1 < E; k1++) x[k1] = cmul(x[k1], twid<DIR, R>(tw, p * k1));
 #pragma unroll
@@ -140,6 +141,9 @@ k_fs_strided(const In* __restrict__ in, StridedAxis ax, const void* twg, Pro pro
 {
     using S = FsShape<R, E, P, fs_threads_strided<R, E, P>()>;
     static_assert(!std::is_same<R, float>::value || S::W >= 8, "a strided tile of fewer than 8 lines");
+    // (radices 5 x 4 have few additions to pack: the y pass of 128 x 200 x 200
+    // with 16-bit spectra takes 105.4 us scalar, 106.6 packed; FP32 127.8, 127.0)
+    constexpr bool PK = E != 20 || sizeof(In) == sizeof(cx<R>);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<R>* tw = reinterpret_cast<cx<R>*>(smem_raw);
     cx<R>* xa = tw + S::L;
@@ -158,14 +162,14 @@ k_fs_strided(const In* __restrict__ in, StridedAxis ax, const void* twg, Pro pro
         x[m] = act ? pro(load_cx(src[(int64_t)j * ax.s]), o, i, j) : mk<R>(0, 0);
     }
     __syncthreads();
-    fs_phase1<R, E, P, DIR>(x, p, xa + w * S::LD, tw);
+    fs_phase1<R, E, P, DIR, PK>(x, p, xa + w * S::LD, tw);
     __syncthreads();
     auto column = [&](int ii) {
         const int k1 = p + P * ii;
         cx<R> u[P];
 #pragma unroll
         for (int q = 0; q < P; q++) u[q] = xa[w * S::LD + k1 * S::KS + q];
-        dft_reg<P, DIR, S::L, R>(u, tw);
+        dft_reg<P, DIR, S::L, R, PK>(u, tw);
         if (act) {
 #pragma unroll
             for (int k2 = 0; k2 < P; k2++) store(u[k2], o, i, k1 + E * k2);
@@ -280,11 +284,27 @@ k_fs_r2c(Src src, int64_t nrows, cx<R>* __restrict__ out, const void* twg)
 
 // inverse complex-to-real rows (2-for-1, see k_c2r_rows), batched: the
 // component index is the fastest grid index.
+// Its first butterfly takes Z = A + i B, formed part by part from two rows,
+// so the packed additions gain little and their register pairs cost moves.
+// us of the x pass, packed / scalar (K = 15): 512 x 64 x 64 FP32 65.8 / 67.9,
+// FP16 70.1 / 70.8; 1024 x 256 x 128 1060 / 1030, 1125 / 1103; 128 x 200 x 200
+// 182 / 176, 172 / 166; 256^3 408 / 415, 464 / 433; 64 x 512 x 512 423 / 403,
+// 421 / 436; 32 x 1024 x 1024 1126 / 1124, 873 / 856. At 1024 in FP32 scalar
+// with 256 threads takes 990.
+template <int E, int P, typename In> constexpr bool fs_c2r_packed()
+{
+    return E == 8 || E * P == (sizeof(In) < sizeof(float2) ? 512 : 256);
+}
+template <typename R, int E, int P, typename In> constexpr int fs_threads_c2r()
+{
+    return P == 32 && sizeof(In) >= sizeof(float2) ? FsThreads<R>::value : fs_threads<R, E, P>();
+}
 template <typename R, int E, int P, class Sink, typename In = cx<R>>
-__global__ void __launch_bounds__((fs_threads<R, E, P>()))
+__global__ void __launch_bounds__((fs_threads_c2r<R, E, P, In>()))
 k_fs_c2r(const In* __restrict__ in, int64_t nrows, Sink sink, const void* twg, int nbatch)
 {
-    using S = FsShape<R, E, P>;
+    using S = FsShape<R, E, P, fs_threads_c2r<R, E, P, In>()>;
+    constexpr bool PK = fs_c2r_packed<E, P, In>();
     constexpr int X = S::L, Xh = X / 2 + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<R>* tw = reinterpret_cast<cx<R>*>(smem_raw);
@@ -310,7 +330,7 @@ k_fs_c2r(const In* __restrict__ in, int64_t nrows, Sink sink, const void* twg, i
         x[m] = k < Xh ? mk<R>(A.x - B.y, A.y + B.x) : mk<R>(A.x + B.y, -A.y + B.x);
     }
     __syncthreads();
-    fs_phase1<R, E, P, +1>(x, p, xa + w * S::LD, tw);
+    fs_phase1<R, E, P, +1, PK>(x, p, xa + w * S::LD, tw);
     __syncthreads();
 #pragma unroll
     for (int ii = 0; ii < E / P; ii++) {
@@ -318,7 +338,7 @@ k_fs_c2r(const In* __restrict__ in, int64_t nrows, Sink sink, const void* twg, i
         cx<R> u[P];
 #pragma unroll
         for (int q = 0; q < P; q++) u[q] = xa[w * S::LD + k1 * S::KS + q];
-        dft_reg<P, +1, S::L, R>(u, tw);
+        dft_reg<P, +1, S::L, R, PK>(u, tw);
 #pragma unroll
         for (int k2 = 0; k2 < P; k2++) {
             const int j = k1 + E * k2;
@@ -542,7 +562,7 @@ inline void launch_c2r_any(const In* in, int64_t nrows, Sink sink, const LenPlan
     if (pl.no_reg || !fs_split(pl.L, E, P)) { launch_c2r_rows<R>(in, nrows, sink, pl, nbatch, st); return; }
 #define TTM_L(E_, P_)                                                                          \
     {                                                                                          \
-        using S = FsShape<R, E_, P_>;                                                          \
+        using S = FsShape<R, E_, P_, fs_threads_c2r<R, E_, P_, In>()>;                         \
         auto k = k_fs_c2r<R, E_, P_, Sink, In>;                                                 \
         set_smem(k, S::SMEM);                                                                  \
         int64_t grid = ceil_div(nrows, 2 * S::W) * nbatch;                                     \
