@@ -409,8 +409,11 @@ __host__ __device__ constexpr size_t p4_smem_bytes()
     return p4_key_bytes(N) + sizeof(float4) * kP4 + sizeof(__half) * (size_t)kP4 * p4_kxs(N);
 }
 
+// CTAs per SM: two by 128 registers, one at n = 6; n = 2 runs no probes and
+// fits 64 registers (24 bytes spilled), and is faster with four than with the
+// three that its free choice of 73 allows: 1.32 -> 1.15 ms on 100 x 256 x 256.
 template <int N>
-__global__ void __launch_bounds__(kP4Threads, N >= 6 ? 1 : 2)
+__global__ void __launch_bounds__(kP4Threads, N >= 6 ? 1 : N == 2 ? 4 : 2)
 k_peakmap4(const float* __restrict__ C, int64_t V, float* __restrict__ score, float* __restrict__ orient,
            float* __restrict__ frob, Probe4Tables tabs)
 {
@@ -770,7 +773,7 @@ void peakmap4_run(ttm_ctx* ctx, int n, const float* C, int64_t V, float* score, 
     // its neighbours, and the SM waits for it with the slots of its other warps
     // empty. 100 x 256 x 256, n = 4, in 8, 16, 32, 64 waves, one block per CTA:
     // 6.05, 5.76, 4.92, 4.29, 4.29 ms; 64 x 128 x 256, n = 6: 6.88, 5.29, 4.19,
-    // 4.30, 4.29 ms. The 66 (101) KB of tables that each CTA copies come from L2.
+    // 4.30, 4.29 ms. The 66 (115) KB of tables that each CTA copies come from L2.
     const int64_t grid = std::min<int64_t>(blocks, (int64_t)1 << 30);
 #define TTM_P4_LAUNCH(N_)                                                                                       \
     {                                                                                                            \

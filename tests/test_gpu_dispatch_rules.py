@@ -63,3 +63,29 @@ def test_register_lengths(T, ctx, shape, prec):
         # three roundings of the storage format (stored spectrum, z- and y-pass stores)
         assert np.linalg.norm(got - C) <= 3 * UNIT[prec] * np.linalg.norm(C)
         assert np.abs(got - C).max() <= 3 * UNIT[prec] * np.abs(C).max()
+
+
+# quaternion maximiser, n = 2 (closed form, its own register budget): less than
+# one voxel block, and a volume of many
+@pytest.mark.parametrize("shape", [(5, 6, 7), (96, 100, 126)])
+def test_quaternion_order2_closed_form(T, ctx, shape):
+    N, V = 5, int(np.prod(shape))
+    field = torch.zeros((10, N, N, N), dtype=torch.float64, device="cuda")
+    field[:, 2, 2, 2] = 1.0
+    plan = T.Plan(ctx, field, T.params(order_n=2, mask_radius=2.0, dprime=4, n_rot_base=1), shape)
+    C = torch.as_tensor(np.random.default_rng(V).standard_normal((10, V)), dtype=torch.float32, device="cuda")
+    s = torch.full(shape, np.nan, device="cuda")
+    q = torch.full((4,) + shape, np.nan, device="cuda")
+    f = torch.full(shape, np.nan, device="cuda")
+    T.ttm_peak_map(plan, C, s, q, f)
+    at = np.unique(np.concatenate([np.arange(max(0, V - 2000), V), np.linspace(0, V - 1, 4000).astype(np.int64)]))
+    c, A = C.cpu().numpy().astype(np.float64)[:, at], np.empty((len(at), 4, 4))
+    for k, (i, j) in enumerate((i, j) for i in range(4) for j in range(i, 4)):
+        A[:, i, j] = A[:, j, i] = c[k]
+    F = np.sqrt((A * A).sum((1, 2)))
+    got, u = s.cpu().numpy().ravel()[at], q.view(4, V).cpu().numpy().astype(np.float64)[:, at].T
+    # sixteen FP32 products of |A| <= F: some 2^-22 F
+    assert np.all(np.abs(got - np.linalg.eigvalsh(A)[:, -1]) <= 1e-5 * F)
+    assert np.all(np.abs(np.einsum("vi,vij,vj->v", u, A, u) - got) <= 1e-5 * F)
+    assert np.all(np.abs(f.cpu().numpy().ravel()[at] - F) <= 1e-6 * F)
+    assert not torch.isnan(s).any() and not torch.isnan(q).any()
