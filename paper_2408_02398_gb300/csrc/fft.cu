@@ -189,6 +189,7 @@ LenPlan make_len_plan(TwiddleCache& tc, int L, int kind)
     TTM_REQUIRE(factor_length(L, pl), E_SHAPE,
                 "transform length " + std::to_string(L) + " is not a product of 2, 3, 5 and 7");
     pl.tw = tc.get(L, kind);
+    pl.num_sms = tc.num_sms;
     return pl;
 }
 

@@ -61,6 +61,7 @@ struct LenPlan {
     int rad[kMaxStages];
     const void* tw;
     uint32_t mag[kMaxStages];  // ceil(2^32 / product of the radices before a stage), set by with_magic
+    int num_sms = 1;  // SMs of the device that runs the passes
     int tile_w = 0;   // lines per CTA of the shared-memory passes (0: default)
     int no_reg = 0;   // 1: use the shared-memory passes even where register kernels exist
 };
@@ -546,6 +547,7 @@ class TwiddleCache {
   public:
     ~TwiddleCache();
     const void* get(int L, int kind);
+    int num_sms = 1;  // of the context's device, handed to the plans
 
   private:
     struct Entry { int L; int kind; void* ptr; };

@@ -320,12 +320,12 @@ k_pfa_zmask(double2* __restrict__ zd, int64_t ncols, const __grid_constant__ Pfa
 // their shared memory, narrowed while fewer than four CTAs per SM remain
 // (every SM's FP64 pipe is the bound, so the CTAs have to spread evenly:
 // 64 x 64 lines in tiles of 16 are 256 CTAs for 152 SMs)
-inline int pfa_tile(int L, int64_t lines, int outer, int min_lw)
+inline int pfa_tile(int num_sms, int L, int64_t lines, int64_t outer, int min_lw)
 {
     auto bytes = [&](int lw) { return ((2ull << lw) + 1) * L * sizeof(double2); };
     int lw = 4;
     while (lw > min_lw && bytes(lw) > 112 * 1024) lw--;
-    while (lw > 2 && ceil_div(lines, 1ll << lw) * outer < 4 * 152) lw--;
+    while (lw > 2 && ceil_div(lines, 1ll << lw) * outer < 4 * (int64_t)num_sms) lw--;
     return lw;
 }
 inline size_t pfa_smem(int L, int lw) { return ((2ull << lw) + 1) * L * sizeof(double2); }
@@ -335,7 +335,7 @@ template <int DIR, class Pro, class Store>
 inline void launch_pfa_strided(const double2* in, StridedAxis ax, const LenPlan& pl, Pro pro, Store store,
                                cudaStream_t st)
 {
-    const int lw = pfa_tile(pl.L, ax.inner, (int)ax.outer, 2);
+    const int lw = pfa_tile(pl.num_sms, pl.L, ax.inner, ax.outer, 2);
     auto k = k_pfa_strided<DIR, Pro, Store>;
     const size_t smem = pfa_smem(pl.L, lw);
     set_smem(k, smem);
@@ -349,7 +349,7 @@ template <int DIR, class Pro, class Store>
 inline void launch_pfa_contig(const double2* in, int64_t nlines, const LenPlan& pl, Pro pro, Store store,
                               cudaStream_t st)
 {
-    const int lw = pfa_tile(pl.L, nlines, 1, 0);
+    const int lw = pfa_tile(pl.num_sms, pl.L, nlines, 1, 0);
     auto k = k_pfa_contig<DIR, Pro, Store>;
     const size_t smem = pfa_smem(pl.L, lw);
     set_smem(k, smem);
@@ -360,7 +360,7 @@ inline void launch_pfa_contig(const double2* in, int64_t nlines, const LenPlan& 
 template <class Mask>
 inline void launch_pfa_zmask(double2* zd, int64_t ncols, const LenPlan& pl, Mask mask, cudaStream_t st)
 {
-    const int lw = pfa_tile(pl.L, ncols, 1, 1);
+    const int lw = pfa_tile(pl.num_sms, pl.L, ncols, 1, 1);
     auto k = k_pfa_zmask<Mask>;
     const size_t smem = pfa_smem(pl.L, lw);
     set_smem(k, smem);

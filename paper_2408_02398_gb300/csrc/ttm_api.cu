@@ -80,6 +80,7 @@ extern "C" ttm_status ttm_ctx_create(int device, ttm_ctx** out)
     try {
         TTM_CUDA_TRY(cudaSetDevice(device));
         TTM_CUDA_TRY(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device));
+        c->twiddles.num_sms = c->num_sms;
         upload_probe_tables(c);
         upload_probe_tables4(c);
         c->peak_scratch = peak_scratch_address();
