@@ -315,8 +315,7 @@ __host__ __device__ constexpr int p4_row(int c, int m)
 
 struct Probe4Tables {
     const float4* dir;    // [kP4] (w, x, y, z), rows as p4_row
-    const __half* phi2h;  // [kP4][p4_kxs(2)] FP16 weighted monomials
-    const __half* phi4h;  // [kP4][p4_kxs(4)]
+    const __half* phi4h;  // [kP4][p4_kxs(4)] FP16 weighted monomials
     const __half* phi6h;  // [kP4][p4_kxs(6)]
     // [kP4] rows of kP4 bits, both in the order 8 cell + member: the second
     // probe (rounded to FP16) is farther than 25 degrees from the first
@@ -638,8 +637,8 @@ k_peakmap4(const float* __restrict__ C, int64_t V, float* __restrict__ score, fl
 // cell is the lowest-index unassigned probe and its 7 nearest unassigned
 // neighbours (distance |q . q'|, as q ~ -q), member m of cell c placed at
 // table row p4_row(c, m). Layout: directions [kP4] float4, then the FP32
-// weighted monomials mult(alpha) q^alpha for n = 2, 4 and 6, [kP4][p4_kp(n)].
-static void build_probe4(std::vector<float>& out, size_t off[4])
+// weighted monomials mult(alpha) q^alpha for n = 4 and 6, [kP4][p4_kp(n)].
+static void build_probe4(std::vector<float>& out, size_t off[3])
 {
     std::vector<double> q;
     rotation_set(kP4, false, q);
@@ -672,7 +671,7 @@ static void build_probe4(std::vector<float>& out, size_t off[4])
     for (int j : src)
         for (int k = 0; k < 4; k++) out.push_back((float)q[4 * j + k]);
     int slot = 1;
-    for (int n : {2, 4, 6}) {
+    for (int n : {4, 6}) {
         off[slot++] = out.size();
         std::vector<int> e;
         exponents4(n, e);
@@ -725,37 +724,32 @@ void upload_probe_tables4(ttm_ctx* ctx)
     TTM_CUDA_TRY(cudaFuncSetAttribute(k_peakmap4<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p4_smem_bytes<4>()));
     TTM_CUDA_TRY(cudaFuncSetAttribute(k_peakmap4<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p4_smem_bytes<6>()));
     std::vector<float> h;
-    size_t off[4];
+    size_t off[3];
     build_probe4(h, off);
     DevBuf f32;
     f32.alloc(h.size() * sizeof(float));
     TTM_CUDA_TRY(cudaMemcpy(f32.p, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice));
     const size_t dir_bytes = sizeof(float4) * kP4;
-    const size_t h2 = sizeof(__half) * (size_t)kP4 * p4_kxs(2), h4 = sizeof(__half) * (size_t)kP4 * p4_kxs(4);
-    const size_t h6 = sizeof(__half) * (size_t)kP4 * p4_kxs(6);
+    const size_t h4 = sizeof(__half) * (size_t)kP4 * p4_kxs(4), h6 = sizeof(__half) * (size_t)kP4 * p4_kxs(6);
     const size_t far_bytes = (size_t)kP4 * kP4 / 8;
-    ctx->probe4.alloc(dir_bytes + h2 + h4 + h6 + far_bytes);
+    ctx->probe4.alloc(dir_bytes + h4 + h6 + far_bytes);
     TTM_CUDA_TRY(cudaMemcpy(ctx->probe4.p, f32.p, dir_bytes, cudaMemcpyDeviceToDevice));
     unsigned char* base = ctx->probe4.as<unsigned char>();
-    k_phi4_half<<<64, 256>>>(f32.as<float>() + off[1], p4_kp(2), ncomp4(2), p4_kxs(2),
+    k_phi4_half<<<64, 256>>>(f32.as<float>() + off[1], p4_kp(4), ncomp4(4), p4_kxs(4),
                              reinterpret_cast<__half*>(base + dir_bytes));
     TTM_LAUNCH_CHECK();
-    k_phi4_half<<<64, 256>>>(f32.as<float>() + off[2], p4_kp(4), ncomp4(4), p4_kxs(4),
-                             reinterpret_cast<__half*>(base + dir_bytes + h2));
-    TTM_LAUNCH_CHECK();
-    k_phi4_half<<<64, 256>>>(f32.as<float>() + off[3], p4_kp(6), ncomp4(6), p4_kxs(6),
-                             reinterpret_cast<__half*>(base + dir_bytes + h2 + h4));
+    k_phi4_half<<<64, 256>>>(f32.as<float>() + off[2], p4_kp(6), ncomp4(6), p4_kxs(6),
+                             reinterpret_cast<__half*>(base + dir_bytes + h4));
     TTM_LAUNCH_CHECK();
     static_assert((sizeof(__half) * kP4) % 16 == 0, "the far table starts on a 16-byte boundary");
     k_far4<<<kP4 * kP4 / 32 / 256, 256>>>(reinterpret_cast<const float4*>(base),
-                                          reinterpret_cast<uint32_t*>(base + dir_bytes + h2 + h4 + h6));
+                                          reinterpret_cast<uint32_t*>(base + dir_bytes + h4 + h6));
     TTM_LAUNCH_CHECK();
     TTM_CUDA_TRY(cudaDeviceSynchronize());
-    ctx->probe4_off[4] = dir_bytes + h2 + h4 + h6;
     ctx->probe4_off[0] = 0;
     ctx->probe4_off[1] = dir_bytes;
-    ctx->probe4_off[2] = dir_bytes + h2;
-    ctx->probe4_off[3] = dir_bytes + h2 + h4;
+    ctx->probe4_off[2] = dir_bytes + h4;
+    ctx->probe4_off[3] = dir_bytes + h4 + h6;
 }
 
 void peakmap4_run(ttm_ctx* ctx, int n, const float* C, int64_t V, float* score, float* orient, float* frob,
@@ -765,8 +759,7 @@ void peakmap4_run(ttm_ctx* ctx, int n, const float* C, int64_t V, float* score, 
     const Probe4Tables t{reinterpret_cast<const float4*>(base + ctx->probe4_off[0]),
                          reinterpret_cast<const __half*>(base + ctx->probe4_off[1]),
                          reinterpret_cast<const __half*>(base + ctx->probe4_off[2]),
-                         reinterpret_cast<const __half*>(base + ctx->probe4_off[3]),
-                         reinterpret_cast<const uint4*>(base + ctx->probe4_off[4])};
+                         reinterpret_cast<const uint4*>(base + ctx->probe4_off[3])};
     const int64_t blocks = std::max<int64_t>(1, ceil_div(V, kP4Threads));
     // One voxel block per CTA (a grid stride beyond the grid's limit): the
     // Newton work of a block varies so much that a CTA of ten ends long after
