@@ -283,9 +283,10 @@ extern "C" ttm_status ttm_refine_peaks(ttm_plan* plan, const float* d_tmpl, cons
         k_pad_template<<<(unsigned)std::min<int64_t>(1024, ceil_div(nt, 256)), 256, 0, st>>>(
             tp64.as<double>(), p.tz, p.ty, p.tx, tp32.as<float2>());
         TTM_LAUNCH_CHECK();
-        // a unit quaternion to 1e-4 scales by as much: 0.02 covers it up to a reach of 126
+        // |q|^2 = 1 - d brings an offset in by up to 2 d of its length: 0.03
+        // covers d = 1e-4 up to a reach of 126, and the rounding of FP32 coordinates
         const std::vector<RefVoxel> list =
-            reach_list(geo, plan->fp.mask_radius + plan->fp.mask_soft_width + std::sqrt(3.0) + 0.02);
+            reach_list(geo, plan->fp.mask_radius + plan->fp.mask_soft_width + std::sqrt(3.0) + 0.03);
         const std::vector<int> offs = ball_offsets(r_s);
         const int n_cand = (int)offs.size() / 3;
         const size_t slots = (size_t)P * n_cand;
