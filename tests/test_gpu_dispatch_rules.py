@@ -89,3 +89,81 @@ def test_quaternion_order2_closed_form(T, ctx, shape):
     assert np.all(np.abs(np.einsum("vi,vij,vj->v", u, A, u) - got) <= 1e-5 * F)
     assert np.all(np.abs(f.cpu().numpy().ravel()[at] - F) <= 1e-6 * F)
     assert not torch.isnan(s).any() and not torch.isnan(q).any()
+
+
+def bf16(a):
+    return torch.as_tensor(np.asarray(a, np.float32)).bfloat16().double().numpy()
+
+
+def gelu(x):
+    return 0.5 * x * (1 + np.tanh(np.sqrt(2 / np.pi) * (x + 0.044715 * x ** 3)))
+
+
+def gelu_grad(x):
+    c = np.sqrt(2 / np.pi)
+    t = np.tanh(c * (x + 0.044715 * x ** 3))
+    return 0.5 * (1 + t) + 0.5 * x * (1 - t * t) * c * (1 + 3 * 0.044715 * x * x)
+
+
+def bf16_loss_grad(p, X, U):
+    """Summed loss and gradient with the operands of every product rounded to BF16, all else in float64."""
+    K, H = X.shape[1], 128
+    at, w = 0, []
+    for s in ((H, K), (H,), (H, H), (H,), (3, H), (3,)):
+        w.append(p[at:at + int(np.prod(s))].reshape(s).astype(np.float64))
+        at += int(np.prod(s))
+    W1, b1, W2, b2, W3, b3 = w
+    a1 = bf16(X) @ bf16(W1).T + b1
+    a2 = bf16(gelu(a1)) @ bf16(W2).T + b2
+    h2 = bf16(gelu(a2))
+    y = h2 @ bf16(W3).T + b3
+    ny = np.linalg.norm(y, axis=1, keepdims=True)
+    u = y / ny
+    dot = (u * U).sum(1, keepdims=True)
+    g = -2 * dot * U
+    dy = (g - (u * g).sum(1, keepdims=True) * u) / ny
+    d2 = bf16(dy) @ bf16(W3) * gelu_grad(a2)
+    d1 = bf16(d2) @ bf16(W2) * gelu_grad(a1)
+    parts = [bf16(d1).T @ bf16(X), d1.sum(0), bf16(d2).T @ bf16(gelu(a1)), d2.sum(0), bf16(dy).T @ h2, dy.sum(0)]
+    return float((1 - dot ** 2).sum()), np.concatenate([v.ravel() for v in parts])
+
+
+# BF16 training products: one row, remainders of the 16-row steps and of the row
+# splits, one and two column tiles of W1, two chunks of rows
+@pytest.mark.parametrize("K,rows", [(6, 1), (15, 63), (28, 65), (28, 4097), (64, 80), (65, 200), (128, 1000),
+                                    (15, 65537)])
+def test_mlp_bf16_gradient_splits(T, ctx, K, rows):
+    rng = np.random.default_rng(K + rows)
+    X = rng.standard_normal((rows, K))
+    U = rng.standard_normal((rows, 3))
+    X = (X / np.linalg.norm(X, axis=1, keepdims=True)).astype(np.float32)
+    U = (U / np.linalg.norm(U, axis=1, keepdims=True)).astype(np.float32)
+    net = T.Mlp(ctx, K, seed=rows)
+    net.set_precision(T.TTM_MLP_BF16)
+    g = torch.full((net.num_params,), np.nan, device="cuda")
+    L = net.loss_grad(dev(X), dev(U), g)
+    Lo, go = bf16_loss_grad(net.get_params(), X, U.astype(np.float64))
+    # FP32 sums, and here and there an operand that FP32 rounds to the
+    # neighbouring BF16 value: 2^-8 of one term of some hundred
+    assert abs(L - Lo) <= 2.0 ** -8 * max(Lo, 1.0)
+    assert np.abs(g.cpu().numpy() - go).max() <= 2.0 ** -8 * np.abs(go).max()
+
+
+# the list of maxima runs out before P peaks are found
+@pytest.mark.parametrize("P,dist", [(1, 1e4), (3000, 0.0), (3000, 7.0), (3000, 1e4)])
+def test_find_peaks_exhausts_its_maxima(T, ctx, P, dist):
+    shape, N = (16, 25, 40), 5
+    m = np.random.default_rng(P).integers(0, 50, shape).astype(np.float32)
+    field = torch.zeros((6, N, N, N), dtype=torch.float64, device="cuda")
+    field[:, 2, 2, 2] = 1.0
+    plan = T.Plan(ctx, field, T.params(order_n=2, mask_radius=2.0, n_rot_base=1), shape)
+    b = plan.valid_box()
+    want_i, want_v = T.ttm_find_peaks_noalloc(ctx, dev(m), b, 16384, 0.0)  # all maxima, in order
+    zyx = np.stack(np.unravel_index(want_i, shape), 1).astype(float)
+    keep = []
+    for k in range(len(want_i)):
+        if len(keep) < P and all(((zyx[k] - zyx[a]) ** 2).sum() >= dist ** 2 for a in keep):
+            keep.append(k)
+    idx, val = T.ttm_find_peaks(plan, dev(m), P, dist)
+    assert idx.tolist() == want_i[keep].tolist() and np.array_equal(val, want_v[keep])
+    assert 0 < len(keep) < max(P, 2)
