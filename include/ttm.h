@@ -500,7 +500,10 @@ void ttm_batch_destroy(ttm_batch* batch);
  * 1 image spectrum, 2 local sums -> w, 3 fused z pass, 4 y pass, 5 x pass
  * with the w epilogue, 6 peak map. ttm_plan_stage_times
  * synchronises, adds the elapsed milliseconds of every call since the last
- * reset into ms[0..n-1] (n <= ttm_num_stages()) and clears the record. */
+ * reset into ms[0..n-1] (n <= ttm_num_stages()) and clears the record.
+ * While it is on, FP64 local sums run in sequence on the stream of the call,
+ * not beside the image spectrum and the z and y passes as in an untimed call
+ * (see ttm_correlate): the stage times add up to a call slower than that. */
 ttm_status ttm_plan_enable_timing(ttm_plan* plan, int on);
 ttm_status ttm_plan_stage_times(ttm_plan* plan, double* ms, int n);
 int ttm_num_stages(void);
