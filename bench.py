@@ -39,11 +39,20 @@ METRIC = "TTM voxels/s (score+orientation map)"
 UNIT = "voxels/s"
 
 
+def code_text(src: str) -> str:
+    """C++ source without its comments, and with one space for each run of
+    white space outside string and character literals."""
+    import re
+    def token(m):
+        return m.group(0) if m.group(0)[0] in "\"'" else " "
+    return re.sub(r'"(?:\\.|[^"\\\n])*"|\'(?:\\.|[^\'\\\n])+\'|(?:\s|//[^\n]*|/\*.*?\*/)+', token, src, flags=re.S).strip()
+
+
 def kernel_sources_digest(entry: str = "") -> str:
-    """SHA-256 over CUDA sources of the library (file names and bytes,
-    sorted), to tell whether a recorded ncu figure still describes them: all
-    of csrc/, or with `entry` (a csrc/ file name) that file and the headers
-    it includes, directly or not."""
+    """SHA-256 over CUDA sources of the library (file names and code, sorted;
+    comments and white space do not count), to tell whether a recorded ncu
+    figure still describes them: all of csrc/, or with `entry` (a csrc/ file
+    name) that file and the headers it includes, directly or not."""
     import glob
     import hashlib
     import re
@@ -64,7 +73,7 @@ def kernel_sources_digest(entry: str = "") -> str:
     h = hashlib.sha256()
     for f in files:
         h.update(os.path.basename(f).encode())
-        h.update(open(f, "rb").read())
+        h.update(code_text(open(f).read()).encode())
     return h.hexdigest()
 
 
