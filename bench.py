@@ -623,14 +623,15 @@ def run_ours(args, ws, rank, local):
     tc_peak = float(pk.get("bf16_tflops", 1900.0))
     pm_flops = 2.0 * K * 128 * V
     tpm = recorded_traffic("traffic_peakmap_n4.md") if n == 4 else None
-    roof_pm = {"bound": "tensor", "kernel": "k_peakmap<%d> (ttm_peak_map)" % n,
+    roof_pm = {"bound": "issue", "kernel": "k_peakmap<%d> (ttm_peak_map)" % n,
                "achieved": pm_flops / (st_ms["peak_map"] / 1e3) / 1e12, "peak": tc_peak, "unit": "TFLOP/s",
                "peak_source": how + " dense BF16 (burst); FP16 mma has the same rate",
                "traffic": None if tpm is None else tpm * V,
                "traffic_source": "profiles/traffic_peakmap_n4.md (ncu dram bytes of one k_peakmap<4> launch on "
                                  "200x256x256, per voxel, scaled to this launch; null once its sources changed)",
                "flops_per_voxel": 2 * K * 128,
-               "note": "issue-bound on the scalar Newton / start work around the probe product",
+               "note": "achieved, peak and frac are the probe product's on the tensor cores; the kernel is bound by "
+                       "instruction issue on the scalar Newton / start work around it (see issue)",
                "warp_inst_per_voxel": recorded_value("k_peakmap_n4_64x512x512.md", "warp_inst_per_voxel") if n == 4
                else None}
     roof_pm["frac"] = roof_pm["achieved"] / roof_pm["peak"]
@@ -908,11 +909,11 @@ def run_quaternion(args):
             "roofline_correlate": {"bound": "hbm", "achieved": alg / (q4["correlate_ms"] / 1e3) / 1e9,
                                    "peak": float(pk.get("hbm_gbs", 6800.0)), "unit": "GB/s", "peak_source": how,
                                    "traffic": None, "bytes_per_voxel": 4 + 4 * K},
-            "roofline_peak_map": {"bound": "tensor", "achieved": probe_flops / (q4["peak_map_ms"] / 1e3) / 1e12,
+            "roofline_peak_map": {"bound": "latency", "achieved": probe_flops / (q4["peak_map_ms"] / 1e3) / 1e12,
                                   "peak": float(pk.get("bf16_tflops", 1900.0)), "unit": "TFLOP/s",
                                   "peak_source": how + " (bf16 dense; the probe product is FP16 mma.sync)",
-                                  "note": "probe-product flops only (2 x %d x 512 per voxel) over the whole maximiser"
-                                          % kx},
+                                  "note": "probe-product flops only (2 x %d x 512 per voxel) over the whole maximiser, "
+                                          "which the latency and issue of the Newton steps bound" % kx},
             "clocks": ck}
     for k in ("roofline_correlate", "roofline_peak_map"):
         line[k]["frac"] = line[k]["achieved"] / line[k]["peak"]
