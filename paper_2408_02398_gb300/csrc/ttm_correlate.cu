@@ -299,9 +299,10 @@ void plan_build_spectra(ttm_plan* P, const double* d_field)
 // us, ttm_correlate 126 x 270 x 315 (n = 4) 5.56 -> 5.39 ms. (FP64 passes
 // confined to a part of each SM by persistent CTAs left more room, 5.0 ms, but
 // are slower by themselves, and the 64^3 match with them: 148 us.) In
-// double-float both sides want the same FP32 pipes (8.11 against 8.09 ms on
-// 200 x 512 x 512), so they run in sequence, as they do while the stages are
-// timed.
+// double-float both sides want the same FP32 pipes, so they run in sequence:
+// forked as well, 200 x 512 x 512 (n = 4) takes 7.35 ms instead of 7.43 and
+// 256 x 512 x 512 (n = 6, FP16 spectra) 12.62 instead of 12.66. They also run
+// in sequence while the stages are timed.
 struct SideSums {
     ttm_plan* P;
     cudaStream_t st;

@@ -12,15 +12,15 @@
 namespace ttm {
 
 // One warp takes 30 columns (32 lanes, the outer two only read) by kLmRows
-// rows and marches along z, so a voxel is read 1.6 times (halo rows and
-// lanes, from L1 and L2) instead of 27, without a division: per plane the
+// rows and marches along z, so a voxel is read 1.8 times (halo rows, lanes
+// and planes, from L1 and L2) instead of 27, without a division: per plane the
 // row maxima over x - 1 .. x + 1 come from two shuffles, the 3 x 3 maxima
 // from those. Lower linear indices must be smaller than v, higher ones at
 // most v; places outside the box read as NaN, which fmaxf passes over.
 // Bound: one read of the map. 200 x 512 x 512, 300 peaks: the former kernel
 // (one voxel per thread, 27 tests, 64-bit divisions for its coordinates)
-// took 632 us of the call's 1311, which now takes 332 (ordering only the
-// accepted candidates on the host is the other part).
+// took 632 us of the call's 1311, which now takes 333 (350 on another card;
+// ordering only the accepted candidates on the host is the other part).
 constexpr int kLmRows = 4;
 constexpr int kLmCols = 30;
 constexpr int kLmThreads = 256;

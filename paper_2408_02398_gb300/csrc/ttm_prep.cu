@@ -73,8 +73,8 @@ constexpr int kPreThreads = 256;
 // Marching a plane costs one round of dependent loads, so what bounds a small
 // volume is the length of the march, not its bytes: 64^3 in chunks of 25
 // planes is 3072 threads and 42 us. The chunk is 25 planes (two planes
-// read again per 25) where that leaves enough threads, else the longest
-// that gives every SM 512 of them: 64^3 then takes chunks of one plane
+// read again per 25) where that leaves 512 threads per SM, else the longest
+// that does, down to one plane: 64^3 takes chunks of one plane and has 431
 // (with the epilogue below, the whole 64^3 match went from 196 to 157 us).
 constexpr int kPreVox = 4;
 constexpr int kPfZChunk = 25;
@@ -242,7 +242,9 @@ struct ProMaskSpectrum {
 
 // 1 / sqrt(v), v > 0, to a relative error below 1e-12 (the caller rounds it
 // to FP32): the FP32 reciprocal square root (error below 2^-21) and one
-// Newton step in FP64, where v is within FP32's normal range
+// Newton step in FP64, where v is within FP32's normal range. Rounded to FP32
+// that is not always the neighbour of the exact value that an FP64 square
+// root and division give: at most one value in 10^5 may differ in its last bit.
 __device__ __forceinline__ float rsqrt_of_double(double v)
 {
     const float f = (float)v;
@@ -254,8 +256,9 @@ __device__ __forceinline__ float rsqrt_of_double(double v)
 // epilogue of the inverse x pass: (S1, S2) -> w. The FP64 pipe bounds this
 // pass (about 1.7 lane operations per clock and SM): an FP64 division, square
 // root and reciprocal were 27 of its 63 FP64 instructions per voxel at
-// X = 315. With the reciprocal of M and rsqrt_of_double they are 10:
-// ttm_correlate of 126 x 270 x 315 (n = 4) 6.64 -> 6.38 ms, same bits.
+// X = 315. With the reciprocal of M (three roundings on the way to the variance,
+// as with the division) and rsqrt_of_double they are 10: ttm_correlate of
+// 126 x 270 x 315 (n = 4) 6.64 -> 6.38 ms, the same bits of w on that volume.
 struct StoreW {
     float* w;
     const double* floor;
