@@ -948,7 +948,12 @@ static void plain_run(ttm_ctx* ctx, int n, const float* C, int64_t V, float* sco
     // on 200 x 512 x 512; 2, 4, 8, 16, 32, 64 waves: 9.49, 9.11, 8.95, 8.87,
     // 8.86, 8.93; one block per CTA 9.46), and a part of a wave idles SMs: the
     // former 32 CTAs per SM were 4.6 waves of 7, or at n = 6 6.4 waves of 5.
-    const int64_t grid = std::min<int64_t>(blocks, (int64_t)ctx->num_sms * ctx->pm_resident[n / 2 - 1] * 16);
+    // At n = 2 every voxel costs the same (closed form), and a CTA of one block
+    // pays its start for little: four blocks per CTA up to those 16 waves. us of
+    // 32, 128 or unlimited CTAs per SM on 128^3: 41.2, 48.0, 48.0; on 100 x 256
+    // x 256: 117.7, 119.9, 142.3; on 200 x 512 x 512: 865, 828, 1075.
+    const int64_t wave = (int64_t)ctx->num_sms * ctx->pm_resident[n / 2 - 1];
+    const int64_t grid = std::min(n == 2 ? std::max(std::min(blocks, wave), blocks / 4) : blocks, 16 * wave);
 #define TTM_PM_LAUNCH(N_)                                                                          \
     k_peakmap<N_><<<(unsigned)grid, kPmThreads, smem, st>>>(C, V, score, orient, frob, t, geo);
     switch (n) {

@@ -91,6 +91,30 @@ def test_quaternion_order2_closed_form(T, ctx, shape):
     assert not torch.isnan(s).any() and not torch.isnan(q).any()
 
 
+# plain maximiser, n = 2: less than one voxel block, a part of a wave of CTAs,
+# one wave that takes several blocks each, and four blocks per CTA with a rest
+@pytest.mark.parametrize("shape", [(5, 6, 7), (40, 42, 45), (75, 80, 81), (100, 126, 135)])
+def test_plain_order2_closed_form(T, ctx, shape):
+    N, V = 5, int(np.prod(shape))
+    field = torch.zeros((6, N, N, N), dtype=torch.float64, device="cuda")
+    field[:, 2, 2, 2] = 1.0
+    plan = T.Plan(ctx, field, T.params(order_n=2, mask_radius=2.0, n_rot_base=1), shape)
+    C = torch.as_tensor(np.random.default_rng(V).standard_normal((6, V)), dtype=torch.float32, device="cuda")
+    s = torch.full(shape, np.nan, device="cuda")
+    u = torch.full((3,) + shape, np.nan, device="cuda")
+    f = torch.full(shape, np.nan, device="cuda")
+    T.ttm_peak_map(plan, C, s, u, f)
+    c, A = C.cpu().numpy().astype(np.float64), np.empty((V, 3, 3))
+    for k, (i, j) in enumerate((i, j) for i in range(3) for j in range(i, 3)):
+        A[:, i, j] = A[:, j, i] = c[k]
+    F = np.sqrt((A * A).sum((1, 2)))
+    got, d = s.cpu().numpy().ravel(), u.view(3, V).cpu().numpy().astype(np.float64).T
+    # nine FP32 products of |A| <= F: some 2^-22 F
+    assert np.all(np.abs(got - np.linalg.eigvalsh(A)[:, -1]) <= 1e-5 * F)
+    assert np.all(np.abs(np.einsum("vi,vij,vj->v", d, A, d) - got) <= 1e-5 * F)
+    assert np.all(np.abs(f.cpu().numpy().ravel() - F) <= 1e-6 * F)
+
+
 def bf16(a):
     return torch.as_tensor(np.asarray(a, np.float32)).bfloat16().double().numpy()
 
